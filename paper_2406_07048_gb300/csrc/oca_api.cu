@@ -41,6 +41,8 @@ struct oca_scene {
     double *d_res = nullptr;
     long long *d_ric_off = nullptr;
     int *d_status = nullptr, *d_iter = nullptr, *d_active = nullptr, *d_err = nullptr;
+    int *d_order = nullptr;     // scenarios by descending horizon [S]
+    int *d_lq_ok = nullptr;     // trajectory step: LQ solve succeeded [S]
     void *d_box = nullptr;      // z_s, w_s [n_states][NSmax]; z_u, w_u [n_ctrls][NUmax]
     int *d_mpc_i = nullptr;     // closed loop: per-step report (iters, status) [2][S]
     double *d_mpc_f = nullptr;  // per-step report (r_pri, r_dual, cost) [3][S] (scene dtype)
@@ -200,8 +202,6 @@ __global__ void k_reset(int *status, int S, int *iter, int *active) {
         *active = S;
     }
 }
-
-__global__ void k_advance(int *iter) { *iter += 1; }
 
 // box block initial state: z = clip(s or u), w = 0 (bounds passed by value)
 template <typename T>
@@ -584,7 +584,7 @@ oca_status admm_impl(oca_scene *sc, const oca_model *m, const oca_admm_params *p
             if (e != cudaSuccess) return e;
         }
         if (prof && (e = rec(cx->ev[2][k])) != cudaSuccess) return e;
-        e = launch_riccati<T>(r, f32, st);
+        e = launch_riccati<T>(r, f32, sc->d_lq_ok, sc->d_order, sc->maxN, cx->n_sm, st);
         if (e != cudaSuccess) return e;
         if (prof && (e = rec(cx->ev[3][k])) != cudaSuccess) return e;
         if (rec_tape) {
@@ -594,8 +594,7 @@ oca_status admm_impl(oca_scene *sc, const oca_model *m, const oca_admm_params *p
             if (e == cudaSuccess) e = tape_box((int)(j + 1));
             if (e != cudaSuccess) return e;
         }
-        k_advance<<<1, 1, 0, st>>>(sc->d_iter);
-        return cudaGetLastError();
+        return cudaSuccess;
     };
     const int G = 8;  // iterations per chunk between host checks
     const long long n_launch = (long long)pr->max_iter + 1;  // j = 0..max_iter
@@ -897,6 +896,8 @@ void free_scene(oca_scene *sc) {
     cudaFree(sc->d_res);
     cudaFree(sc->d_ric_off);
     cudaFree(sc->d_status);
+    cudaFree(sc->d_order);
+    cudaFree(sc->d_lq_ok);
     cudaFree(sc->d_mpc_i);
     cudaFree(sc->d_rev_iters);
     cudaFree(sc->d_mpc_f);
@@ -1081,6 +1082,10 @@ oca_status oca_scene_create(oca_ctx *ctx, const oca_scene_desc *d, oca_scene **o
             const int cols = sc->meta[s].NP * sc->meta[s].N - 32 * k;
             tl.push_back(Tile{s, 32 * k, cols <= 16 ? 1 : 0});
         }
+    // the trajectory step pairs scenarios of about the same horizon, longest first
+    std::vector<int> by_horizon(S);
+    for (int s = 0; s < S; ++s) by_horizon[s] = s;
+    std::stable_sort(by_horizon.begin(), by_horizon.end(), [&](int x, int y) { return sc->meta[x].N > sc->meta[y].N; });
     // warps per tile: about 8 obstacles per warp at the median obstacle count
     std::nth_element(Ms.begin(), Ms.begin() + Ms.size() / 2, Ms.end());
     const int Mmed = Ms[Ms.size() / 2];
@@ -1112,6 +1117,8 @@ oca_status oca_scene_create(oca_ctx *ctx, const oca_scene_desc *d, oca_scene **o
         (e = dmalloc(&sc->d_ric_off, sizeof(long long) * S)) != OCA_OK ||
         (e = dmalloc(&sc->d_res, sizeof(double) * 4 * (size_t)tiles)) != OCA_OK ||
         (e = dmalloc(&sc->d_status, sizeof(int) * S)) != OCA_OK ||
+        (e = dmalloc(&sc->d_order, sizeof(int) * S)) != OCA_OK ||
+        (e = dmalloc(&sc->d_lq_ok, sizeof(int) * S)) != OCA_OK ||
         (e = dmalloc(&sc->d_mpc_i, sizeof(int) * 2 * S)) != OCA_OK ||
         (e = dmalloc(&sc->d_rev_iters, sizeof(int) * S)) != OCA_OK ||
         (e = dmalloc(&sc->d_mpc_f, sizeof(double) * 3 * S)) != OCA_OK ||
@@ -1134,6 +1141,7 @@ oca_status oca_scene_create(oca_ctx *ctx, const oca_scene_desc *d, oca_scene **o
               cudaMemcpy(sc->d_obs_nf, d->obs_nf, sizeof(int) * M_tot, cudaMemcpyHostToDevice) == cudaSuccess &&
               cudaMemcpy(sc->d_part_nf, d->part_nf, sizeof(int) * P_tot, cudaMemcpyHostToDevice) == cudaSuccess &&
               cudaMemcpy(sc->d_part_link, d->part_link, sizeof(int) * P_tot, cudaMemcpyHostToDevice) == cudaSuccess &&
+              cudaMemcpy(sc->d_order, by_horizon.data(), sizeof(int) * S, cudaMemcpyHostToDevice) == cudaSuccess &&
               cudaMemcpy(sc->d_ric_off, roff.data(), sizeof(long long) * S, cudaMemcpyHostToDevice) == cudaSuccess &&
               cudaMemset(sc->d_err, 0, sizeof(int)) == cudaSuccess &&
               cudaMemset(sc->d_res, 0, sizeof(double) * 4 * (size_t)tiles) == cudaSuccess;

@@ -224,7 +224,7 @@ struct RicArgs {
     T *box_zu, *box_wu;  // [n_ctrls][NU]
     double *box_res;     // [S][2] box residuals of the last trajectory step
     int max_iter;
-    const int *iter;
+    int *iter;
     const T *s_ref;
     T *s;
     T *u;

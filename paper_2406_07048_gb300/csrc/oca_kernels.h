@@ -22,8 +22,11 @@ cudaError_t launch_scale(const ScaleArgs<T> &a, int dim, int n_tiles, int W, cud
 template <typename T>
 cudaError_t launch_cert(const CertArgs<T> &a, int n_tiles, int W, cudaStream_t st);
 
+// trajectory step and the advance of the iteration counter; lq_ok: [S] work array,
+// order: scenarios by descending horizon, max_n the longest
 template <typename T>
-cudaError_t launch_riccati(const RicArgs<T> &a, bool f32, cudaStream_t st);
+cudaError_t launch_riccati(const RicArgs<T> &a, bool f32, int *lq_ok, const int *order, int max_n, int n_sm,
+                           cudaStream_t st);
 
 long long riccati_scratch_elems(int kind, int N);
 

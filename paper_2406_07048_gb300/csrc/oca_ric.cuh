@@ -154,13 +154,13 @@ struct StageParams {
     int Qtot;
 };
 
-// Stage t of one scenario into the factorisation-precision scratch:
-// A_t, B_t, c_t, r_t (t < N) and Q_t, q_t (t <= N); assembled in T.
-template <typename T, typename F, int KIND>
-__device__ void assemble_stage(const StageParams<T> &a, const StageSrc<T> &src, const ScenMeta &sm, int t, F *scr) {
+// Stage t of one scenario, assembled in T: A_t, B_t, c_t, r_t (t < N) and Q_t,
+// q_t (t <= N) go to a sink (out.A(i, k, v), out.B, out.c, out.u for r_t, out.Q, out.q), which stores them
+// in the factorisation precision.
+template <typename T, int KIND, class Sink>
+__device__ void assemble_terms(const StageParams<T> &a, const StageSrc<T> &src, const ScenMeta &sm, int t, Sink &out) {
     constexpr int NS = MDims<KIND>::NS, NU = MDims<KIND>::NU, D = MDims<KIND>::D;
     constexpr int NW = StatDims<D>::NW;
-    using LY = RicLayout<NS, NU>;
     const int N = sm.N;
     const DevModel<T> &mdt = a.model;
     T st[NS];
@@ -171,20 +171,22 @@ __device__ void assemble_stage(const StageParams<T> &a, const StageSrc<T> &src, 
 #pragma unroll
         for (int i = 0; i < NU; ++i) ut[i] = src.u[(long long)(sm.ctrl0 + t) * NU + i];
         dynamics<T, KIND>(mdt, st, ut, f, fs, fu);
-        F *At = scr + LY::A(N, t), *Bt = scr + LY::B(N, t), *ct = scr + LY::c(N, t), *rt = scr + LY::r(N, t);
+#pragma unroll
         for (int i = 0; i < NS; ++i) {
             T acc = st[i] + mdt.dt * f[i];
+#pragma unroll
             for (int k = 0; k < NS; ++k) {
                 const T v = (i == k ? T(1) : T(0)) + mdt.dt * fs[i * NS + k];
-                At[i * NS + k] = F(v);
+                out.A(i, k, v);
                 acc -= v * st[k];
             }
+#pragma unroll
             for (int k = 0; k < NU; ++k) {
                 const T v = mdt.dt * fu[i * NU + k];
-                Bt[i * NU + k] = F(v);
+                out.B(i, k, v);
                 acc -= v * ut[k];
             }
-            ct[i] = F(acc);
+            out.c(i, acc);
         }
         // control linear term: damping toward u^j, box block
 #pragma unroll
@@ -192,7 +194,7 @@ __device__ void assemble_stage(const StageParams<T> &a, const StageSrc<T> &src, 
             const long long k2 = (long long)(sm.ctrl0 + t) * NU + i;
             T acc = -a.damp * ut[i];
             if (bounded(mdt.u_lo[i], mdt.u_hi[i])) acc -= a.rho_box * (src.zu[k2] - src.wu[k2]);
-            rt[i] = F(acc);
+            out.u(i, acc);
         }
     }
     T Qr[NS * NS], qr[NS];
@@ -236,10 +238,32 @@ __device__ void assemble_stage(const StageParams<T> &a, const StageSrc<T> &src, 
             }
         }
     }
-    F *Qt = scr + LY::Q(N, t), *qt = scr + LY::q(N, t);
-    for (int i = 0; i < NS * NS; ++i) Qt[i] = F(Qr[i]);
-    for (int i = 0; i < NS; ++i) qt[i] = F(qr[i]);
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+#pragma unroll
+        for (int k = 0; k < NS; ++k) out.Q(i, k, Qr[i * NS + k]);
+        out.q(i, qr[i]);
+    }
 }
+
+// the dense scratch (RicLayout) in the factorisation precision
+template <typename T, typename F, int KIND>
+__device__ void assemble_stage(const StageParams<T> &a, const StageSrc<T> &src, const ScenMeta &sm, int t, F *scr) {
+    constexpr int NS = MDims<KIND>::NS, NU = MDims<KIND>::NU;
+    using LY = RicLayout<NS, NU>;
+    struct Sink {
+        F *At, *Bt, *ct, *rt, *Qt, *qt;
+        __device__ void A(int i, int k, T v) { At[i * NS + k] = F(v); }
+        __device__ void B(int i, int k, T v) { Bt[i * NU + k] = F(v); }
+        __device__ void c(int i, T v) { ct[i] = F(v); }
+        __device__ void u(int i, T v) { rt[i] = F(v); }
+        __device__ void Q(int i, int k, T v) { Qt[i * NS + k] = F(v); }
+        __device__ void q(int i, T v) { qt[i] = F(v); }
+    } out{scr + LY::A(sm.N, t), scr + LY::B(sm.N, t), scr + LY::c(sm.N, t), scr + LY::r(sm.N, t),
+          scr + LY::Q(sm.N, t), scr + LY::q(sm.N, t)};
+    assemble_terms<T, KIND>(a, src, sm, t, out);
+}
+
 
 // ----------------------------------------------------------------------------
 // Backward Riccati recursion over the scratch (one warp; every lane calls):

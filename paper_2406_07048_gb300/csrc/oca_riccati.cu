@@ -5,7 +5,7 @@
 // problem (Riccati) with the augmented term 0.5 rho_b |(s,u) - z + w|^2; a
 // proximal term 0.5 damp |(s,u) - (s,u)^j|^2 damps the SQP step.
 //
-// One warp per scenario.  At launch j the warp
+// At launch j every scenario
 //   1. tests the stopping rule of iteration j-1 (Sec. IV-B):
 //        r_pri  = sum dzeta^2 + |dxi|^2     (partials written by the pair kernel's head at j)
 //        r_dual = sum |dlambda|^2 + |dmu|^2 (partials written by the pair kernel at j-1)
@@ -16,16 +16,23 @@
 //      per-(part, t) statistics W, Wc, E through the pose Jacobians;
 //   3. runs the backward Riccati recursion (factorisation precision F) and
 //      the forward sweep, writing s^{j+1}, u^{j+1} and the new poses.
+// The 2-D models run as three kernels (below), the 12-state model as one kernel
+// with a four-warp CTA per scenario.
+#include <algorithm>
+#include <type_traits>
+
 #include "oca_common.cuh"
 #include "oca_kernels.h"
 #include "oca_ric.cuh"
+#include "oca_ricprog.cuh"
 
 namespace oca {
 
 long long riccati_scratch_elems(int kind, int N) {
     switch (kind) {
-        case 0: return RicLayout<4, 2>::size(N);
-        case 1: return RicLayout<5, 2>::size(N);
+        // the forward step's packed records and the adjoint's dense layout share the block
+        case 0: return std::max(RicLayout<4, 2>::size(N), RicMap<0>::size(N));
+        case 1: return std::max(RicLayout<5, 2>::size(N), RicMap<1>::size(N));
         default: return RicLayout<12, 4>::size(N);
     }
 }
@@ -58,6 +65,107 @@ __device__ void finish_scenario(const RicArgs<T> &a, const ScenMeta &sm, int s, 
     }
 }
 
+// stopping rule of iteration j-1 (one warp): true when the scenario is done
+template <typename T, int KIND>
+__device__ bool stop_rule(const RicArgs<T> &a, const ScenMeta &sm, int s, int j) {
+    const int lane = threadIdx.x;
+    if (j >= 1) {
+        const double *rcur = a.res + (size_t)(j & 1) * a.n_tiles * 2;
+        const double *rprev = a.res + (size_t)((j - 1) & 1) * a.n_tiles * 2;
+        double rp = 0.0, rd = 0.0;
+        for (int k = lane; k < sm.ntile; k += 32) {
+            rp += rcur[(size_t)(sm.tile0 + k) * 2];
+            rd += rprev[(size_t)(sm.tile0 + k) * 2 + 1];
+        }
+        rp = warp_sum(rp) + a.box_res[2 * s];      // + box-block residuals of iteration j-1
+        rd = warp_sum(rd) + a.box_res[2 * s + 1];
+        const bool conv = rp <= double(a.eps_pri) && rd <= double(a.eps_dual);
+        if (conv || j >= a.max_iter) {
+            finish_scenario<T, KIND>(a, sm, s, conv ? OCA_SCEN_CONVERGED : OCA_SCEN_MAX_ITER, j, rp, rd);
+            return true;
+        }
+    } else if (a.max_iter <= 0) {
+        finish_scenario<T, KIND>(a, sm, s, OCA_SCEN_MAX_ITER, 0, 0.0, 0.0);
+        return true;
+    }
+    return false;
+}
+
+template <typename T>
+__device__ __forceinline__ void stage_inputs(const RicArgs<T> &a, StageParams<T> &sp, StageSrc<T> &src) {
+    sp.model = a.model;
+    sp.g = a.g;
+    sp.sigma = a.sigma;
+    sp.rho_box = a.rho_box;
+    sp.damp = a.damp;
+    sp.s_ref = a.s_ref;
+    sp.Qtot = a.Qtot;
+    src.s = a.s;
+    src.u = a.u;
+    src.zs = a.box_zs;
+    src.ws = a.box_ws;
+    src.zu = a.box_zu;
+    src.wu = a.box_wu;
+    src.stats = a.stats;
+}
+
+// Step t of the new iterate (st = s_{t+1}, ut = u_t as stored): box block
+// z = clip(x + w), w += x - z of its components, poses of s_{t+1}.  Everything is
+// loaded before the first store: each load costs most of a microsecond and the
+// compiler may not move one past a store.
+template <typename T, int KIND>
+__device__ __forceinline__ void box_poses(const RicArgs<T> &a, const ScenMeta &sm, int t, const T *st, const T *ut, double &rpb,
+                                          double &rdb) {
+    constexpr int NS = MDims<KIND>::NS, NU = MDims<KIND>::NU, D = MDims<KIND>::D;
+    const long long ks = (long long)(sm.state0 + t + 1) * NS, ku = (long long)(sm.ctrl0 + t) * NU;
+    const bool box = a.rho_box > T(0);  // rho_box = 0: no box block
+    T zs[NS], ws[NS], zu[NU], wu[NU];
+    bool bs[NS], bu[NU];
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        bs[i] = box && bounded(a.model.s_lo[i], a.model.s_hi[i]);
+        if (bs[i]) {
+            zs[i] = a.box_zs[ks + i];
+            ws[i] = a.box_ws[ks + i];
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < NU; ++i) {
+        bu[i] = box && bounded(a.model.u_lo[i], a.model.u_hi[i]);
+        if (bu[i]) {
+            zu[i] = a.box_zu[ku + i];
+            wu[i] = a.box_wu[ku + i];
+        }
+    }
+    for (int part = 0; part < sm.NP; ++part) {
+        const int gp = sm.part0 + part;
+        T off[D], rho[D], R[D * D];
+#pragma unroll
+        for (int i = 0; i < D; ++i) off[i] = ldg(a.g.part_off + gp * D + i);
+        part_pose<T, KIND>(a.model, ldg(a.g.part_link + gp), off, st, rho, R, nullptr, nullptr, nullptr);
+        const int col = sm.qbeg + part * sm.N + t;
+#pragma unroll
+        for (int i = 0; i < D; ++i) a.pose[(long long)i * a.Qtot + col] = rho[i];
+#pragma unroll
+        for (int i = 0; i < D * D; ++i) a.pose[(long long)(D + i) * a.Qtot + col] = R[i];
+    }
+    auto update = [&](T x, T lo, T hi, T z, T w, T *zo, T *wo) {
+        const T zn = fmin(fmax(x + w, lo), hi);
+        rdb += double(zn - z) * double(zn - z);
+        rpb += double(x - zn) * double(x - zn);
+        *zo = zn;
+        *wo = w + (x - zn);
+    };
+#pragma unroll
+    for (int i = 0; i < NS; ++i)
+        if (bs[i]) update(st[i], a.model.s_lo[i], a.model.s_hi[i], zs[i], ws[i], a.box_zs + ks + i, a.box_ws + ks + i);
+#pragma unroll
+    for (int i = 0; i < NU; ++i)
+        if (bu[i]) update(ut[i], a.model.u_lo[i], a.model.u_hi[i], zu[i], wu[i], a.box_zu + ku + i, a.box_wu + ku + i);
+}
+
+__global__ void k_advance(int *iter) { *iter += 1; }
+
 // NT threads per scenario: warp 0 runs every phase but the Riccati
 // recursion, which all NT threads share (NT > 32 for the 12-state model,
 // whose per-step products have 150-200 entries).
@@ -75,26 +183,8 @@ __global__ void __launch_bounds__(NT) k_riccati(RicArgs<T> a) {
 
     // ---- 1. stopping rule of iteration j-1 (warp 0)
     if (lane < 32) {
-        s_retired = 0;
-    if (j >= 1) {
-        const double *rcur = a.res + (size_t)(j & 1) * a.n_tiles * 2;
-        const double *rprev = a.res + (size_t)((j - 1) & 1) * a.n_tiles * 2;
-        double rp = 0.0, rd = 0.0;
-        for (int k = lane; k < sm.ntile; k += 32) {
-            rp += rcur[(size_t)(sm.tile0 + k) * 2];
-            rd += rprev[(size_t)(sm.tile0 + k) * 2 + 1];
-        }
-        rp = warp_sum(rp) + a.box_res[2 * s];      // + box-block residuals of iteration j-1
-        rd = warp_sum(rd) + a.box_res[2 * s + 1];
-        const bool conv = rp <= double(a.eps_pri) && rd <= double(a.eps_dual);
-        if (conv || j >= a.max_iter) {
-            finish_scenario<T, KIND>(a, sm, s, conv ? OCA_SCEN_CONVERGED : OCA_SCEN_MAX_ITER, j, rp, rd);
-            s_retired = 1;
-        }
-    } else if (a.max_iter <= 0) {
-        finish_scenario<T, KIND>(a, sm, s, OCA_SCEN_MAX_ITER, 0, 0.0, 0.0);
-        s_retired = 1;
-    }
+        const bool r = stop_rule<T, KIND>(a, sm, s, j);
+        if (lane == 0) s_retired = r;
     }
     ric_sync<NT>();
     if (s_retired) return;
@@ -104,21 +194,8 @@ __global__ void __launch_bounds__(NT) k_riccati(RicArgs<T> a) {
     // ---- 2. stage assembly, lanes over t (in the array precision T; only
     // the factorisation below runs in F)
     StageParams<T> sp;
-    sp.model = a.model;
-    sp.g = a.g;
-    sp.sigma = a.sigma;
-    sp.rho_box = a.rho_box;
-    sp.damp = a.damp;
-    sp.s_ref = a.s_ref;
-    sp.Qtot = a.Qtot;
     StageSrc<T> src;
-    src.s = a.s;
-    src.u = a.u;
-    src.zs = a.box_zs;
-    src.ws = a.box_ws;
-    src.zu = a.box_zu;
-    src.wu = a.box_wu;
-    src.stats = a.stats;
+    stage_inputs(a, sp, src);
     for (int t = lane; t <= N; t += NT) assemble_stage<T, F, KIND>(sp, src, sm, t, scr);
     ric_sync<NT>();
 
@@ -203,24 +280,433 @@ __global__ void __launch_bounds__(NT) k_riccati(RicArgs<T> a) {
     }
 }
 
-template <typename T, typename F>
-cudaError_t launch_riccati_f(const RicArgs<T> &a, cudaStream_t st) {
-    switch (a.model.kind) {
-        case 0: k_riccati<T, F, 0, 32><<<a.n_scen, 32, 0, st>>>(a); break;
-        case 1: k_riccati<T, F, 1, 32><<<a.n_scen, 32, 0, st>>>(a); break;
-        case 2: k_riccati<T, F, 2, 128><<<a.n_scen, 128, 0, st>>>(a); break;
-        default: return cudaErrorInvalidValue;
+// ============================================================================
+// 2-D models: three kernels per trajectory step.
+//   k_traj_stage   stopping rule and stage assembly, lanes over t (FP32 work with
+//                  everything in registers, written as one packed record per stage)
+//   k_traj_lq      backward recursion and forward sweep (the FP64 chain), L lanes
+//                  per scenario, 32 / L scenarios per warp
+//   k_traj_apply   the new iterate in T, box block and poses, lanes over t
+// The recursion is bound by FP64 issue (oca_ricprog.cuh), the other two by latency;
+// apart, the recursion keeps one warp per scheduler busy with nothing but the
+// recursion, and the assembly and the box block run over all horizon steps at once.
+// 2,048 trailer scenarios, mean horizon 50: 34 + 138 + 18 us per step; one warp
+// per scenario doing everything with dense products took 510 us.  A stage of the
+// recursion takes 2,660 cycles (22 FP64 instructions: 1,408 of them), a step of the
+// sweep 700; the 80-stage scenarios set the time.
+// ============================================================================
+
+// the lists of multiply-adds of the recursion's three products
+template <int KIND, int L, int PHASE>
+__device__ constexpr auto kRicTab = RicBuild<KIND>::template table<PHASE, L>();
+template <int KIND>
+__device__ constexpr auto kRicOut = RicBuild<KIND>::out_map();
+
+// 1 / x by one step of the third-order Newton-Schulz iteration
+// y <- y + y (e + e^2), e = 1 - x y, from the hardware's approximation: the error
+// e (about 2^-20) becomes e^3 < 2^-53 with three multiply-adds
+__device__ __forceinline__ double lq_rcp(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ float lq_rcp(float x) { return 1.0f / x; }
+// x > 0 and x finite on the integer pipe (an FP64 compare costs as much as a multiply-add)
+__device__ __forceinline__ bool lq_positive(double x) {
+    const long long b = __double_as_longlong(x);
+    return b > 0 && b <= 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool lq_positive(float x) { return x > 0.0f; }
+__device__ __forceinline__ bool lq_finite(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) != 0x7ff; }
+__device__ __forceinline__ bool lq_finite(float x) { return isfinite(x); }
+
+// 8- or 4-byte access at a shared-memory byte address
+__device__ __forceinline__ double lds(unsigned at, double) {
+    double v;
+    asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(at) : "memory");
+    return v;
+}
+__device__ __forceinline__ float lds(unsigned at, float) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(at) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts(unsigned at, double v) { asm volatile("st.shared.f64 [%0], %1;" ::"r"(at), "d"(v) : "memory"); }
+__device__ __forceinline__ void sts(unsigned at, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(at), "f"(v) : "memory"); }
+
+// One product's slots of one lane: the four shared-memory addresses of each slot,
+// decoded once (a warp alone on its scheduler pays several cycles for every
+// instruction, so the step decodes nothing).
+template <typename F, int SLOTS>
+struct LqSlots {
+    unsigned in[SLOTS], c[SLOTS], v[SLOTS], st[SLOTS];
+    unsigned cont;  // bit i: slot i continues the accumulator of slot i - 1
+
+    template <int L>
+    __device__ __forceinline__ void load(const RicPhase<SLOTS, L> &tab, int lane, const F *region) {
+        const unsigned base = (unsigned)__cvta_generic_to_shared(region);
+        cont = 0;
+#pragma unroll
+        for (int i = 0; i < SLOTS; ++i) {
+            const uint64_t w = tab.code[i][lane];
+            const unsigned at = (unsigned)w & 0xffffu;
+            const bool k = at == (unsigned)kRicCont;
+            cont |= (k ? 1u : 0u) << i;
+            in[i] = base + (k ? 0u : at) * (unsigned)sizeof(F);
+            c[i] = base + ((unsigned)(w >> 16) & 0xffffu) * (unsigned)sizeof(F);
+            v[i] = base + ((unsigned)(w >> 32) & 0xffffu) * (unsigned)sizeof(F);
+            st[i] = base + ((unsigned)(w >> 48) & 0xffffu) * (unsigned)sizeof(F);
+        }
     }
+    // A product reads nothing that it writes, so all operands are loaded first and
+    // the multiply-adds follow each other without a load's latency between them.
+    __device__ __forceinline__ void run() const {
+        F a[SLOTS], x[SLOTS], y[SLOTS];
+#pragma unroll
+        for (int i = 0; i < SLOTS; ++i) {
+            a[i] = lds(in[i], F(0));
+            x[i] = lds(c[i], F(0));
+            y[i] = lds(v[i], F(0));
+        }
+#pragma unroll
+        for (int i = 0; i < SLOTS; ++i) a[i] = fma(x[i], y[i], i > 0 && (cont >> i & 1u) ? a[i > 0 ? i - 1 : 0] : a[i]);
+#pragma unroll
+        for (int i = 0; i < SLOTS; ++i) sts(st[i], a[i]);
+    }
+};
+template <typename F, class Tab>
+struct LqSlotsOf;
+template <typename F, int SLOTS, int L>
+struct LqSlotsOf<F, RicPhase<SLOTS, L>> {
+    using type = LqSlots<F, SLOTS>;
+};
+
+// threads per scenario of the per-step kernels: one per horizon step up to 96
+constexpr int kTrajBlock = 96;
+template <typename F, int KIND>
+constexpr int traj_rec_stride() { return RicMap<KIND>::REC | 1; }
+
+template <typename T, typename F, int KIND>
+__global__ void __launch_bounds__(kTrajBlock) k_traj_stage(RicArgs<T> a) {
+    constexpr int NS = MDims<KIND>::NS;
+    using Mp = RicMap<KIND>;
+    const int s = blockIdx.x, lane = threadIdx.x, NT = blockDim.x;
+    if (a.scen_status[s] != kActive) return;
+    const int j = *a.iter;
+    if (j > a.max_iter) return;
+    const ScenMeta sm = a.meta[s];
+    __shared__ int s_retired;
+    if (lane < 32) {
+        const bool r = stop_rule<T, KIND>(a, sm, s, j);
+        if (lane == 0) s_retired = r;
+    }
+    __syncthreads();
+    if (s_retired) return;
+    F *scr = reinterpret_cast<F *>(a.scratch) + a.scratch0[s];
+    StageParams<T> sp;
+    StageSrc<T> src;
+    stage_inputs(a, sp, src);
+    struct Sink {
+        F *r;
+        __device__ void A(int i, int k, T v) {
+            const int e = RicSparse<KIND>::a_slot(i, k);
+            if (e >= 0) r[Mp::rA + e] = F(v);
+        }
+        __device__ void B(int i, int k, T v) {
+            const int e = RicSparse<KIND>::b_slot(i, k);
+            if (e >= 0) r[Mp::rB + e] = F(v);
+        }
+        __device__ void c(int i, T v) { r[Mp::rc + i] = F(v); }
+        __device__ void u(int i, T v) { r[Mp::rr + i] = F(v); }
+        __device__ void Q(int i, int k, T v) {
+            if (i <= k) r[Mp::rQ + Mp::sym(i, k)] = F(v);
+        }
+        __device__ void q(int i, T v) { r[Mp::rq + i] = F(v); }
+    };
+    // records through shared memory (odd stride): written straight to the scratch,
+    // every 8-byte store of a warp touches 32 sectors
+    constexpr int RS = traj_rec_stride<F, KIND>();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    F *rec = reinterpret_cast<F *>(smem_raw);  // [NT][RS]
+    for (int t0 = 0; t0 <= sm.N; t0 += NT) {
+        const int n = min(NT, sm.N + 1 - t0);
+        if (lane < n) {
+            Sink out{rec + lane * RS};
+            assemble_terms<T, KIND>(sp, src, sm, t0 + lane, out);
+        }
+        __syncthreads();
+        F *dst = scr + Mp::rec(t0);
+        for (int e = lane; e < n * Mp::REC; e += NT) dst[e] = rec[e / Mp::REC * RS + e % Mp::REC];
+        __syncthreads();
+    }
+    if (lane < NS) scr[Mp::s0(sm.N) + lane] = F(a.s[(long long)sm.state0 * NS + lane]);
+}
+
+// What the recursion needs of a launch, free of the array type T.
+template <typename F>
+struct LqArgs2 {
+    const ScenMeta *meta;
+    const int *order;        // scenarios by descending horizon
+    int n_scen;
+    const int *scen_status;
+    void *scratch;
+    const long long *scratch0;
+    F dt, ru[4];
+    int *ok;                 // [S] out: factorisation and sweep finite and positive definite
+    int *iter;               // advanced by one
+};
+
+// One CTA per SM, two warps per scheduler.  A group of 32 / L scenarios (neighbours
+// in the order, so of about the same horizon) takes one warp, L lanes each; the
+// groups, longest first, are dealt to the K = 4 x CTAs schedulers back and forth
+// (0..K-1, K-1..0, ...), so that the longest chains have a scheduler for themselves
+// and the others share with short ones: two long chains on one scheduler would each
+// run at half speed.  Per stage: the three products as slot lists, the 2 x 2
+// inverse between them, the next record loaded meanwhile.  F = A + B K and f = c + B k
+// are formed with P, by lanes that would otherwise idle, so that the sweep is one
+// matrix-vector product per step (lane i owns s_i) instead of two dependent ones.
+constexpr int kLqWarps = 8;
+template <typename F, int KIND, int L>
+__global__ void __launch_bounds__(32 * kLqWarps) k_traj_lq(LqArgs2<F> a) {
+    using Mp = RicMap<KIND>;
+    constexpr int NS = Mp::NS, NU = Mp::NU, G = 32 / L, REC = Mp::REC, OUT = Mp::OUT;
+    static_assert(NU == 2, "2-D models");
+    constexpr int PR = (REC + L - 1) / L, PO = (OUT + L - 1) / L, KE = NU * (NS + 1), PK = (KE + L - 1) / L;
+    __shared__ F region[kLqWarps][G][Mp::SIZE];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane / L, li = lane % L;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.iter += 1;
+    const int n_group = (a.n_scen + G - 1) / G, K = 4 * gridDim.x, slot = (warp & 3) * gridDim.x + blockIdx.x;
+    F *sm = region[warp][g];
+
+    typename LqSlotsOf<F, std::remove_cv_t<decltype(kRicTab<KIND, L, 0>)>>::type prod_y;
+    typename LqSlotsOf<F, std::remove_cv_t<decltype(kRicTab<KIND, L, 1>)>>::type prod_m;
+    typename LqSlotsOf<F, std::remove_cv_t<decltype(kRicTab<KIND, L, 2>)>>::type prod_p;
+    prod_y.load(kRicTab<KIND, L, 0>, li, sm);
+    prod_m.load(kRicTab<KIND, L, 1>, li, sm);
+    prod_p.load(kRicTab<KIND, L, 2>, li, sm);
+    int om[PO];
+#pragma unroll
+    for (int r = 0; r < PO; ++r) om[r] = li + L * r < OUT ? kRicOut<KIND>.at[li + L * r] : 0;
+
+    if (li == 0) {
+        sm[Mp::ZERO] = F(0);
+        sm[Mp::ONE] = F(1);
+        sm[Mp::DT] = a.dt;
+        for (int x = 0; x < NU; ++x) sm[Mp::RU + x] = a.ru[x];
+    }
+    for (int round = warp >> 2; round * K < n_group; round += kLqWarps / 4) {
+    const int group = round & 1 ? (round + 1) * K - 1 - slot : round * K + slot;
+    const int at = group * G + g;
+    const int s = group < n_group && at < a.n_scen ? a.order[at] : -1;
+    const bool live = s >= 0 && a.scen_status[s] == kActive;
+    if (!__any_sync(0xffffffffu, live)) continue;
+    const int N = live ? a.meta[s].N : 0;
+    int Nm = N;
+#pragma unroll
+    for (int o = 16; o >= L; o >>= 1) Nm = max(Nm, __shfl_xor_sync(0xffffffffu, Nm, o));
+    F *scr = reinterpret_cast<F *>(a.scratch) + (live ? a.scratch0[s] : 0);
+    __syncwarp();
+    if (live) {
+        const F *rN = scr + Mp::rec(N), *r1 = scr + Mp::rec(N - 1);
+        for (int e = li; e < Mp::NSYM; e += L) sm[Mp::P0 + e] = rN[Mp::rQ + e];
+        for (int e = li; e < NS; e += L) sm[Mp::p0 + e] = rN[Mp::rq + e];
+        for (int e = li; e < REC; e += L) sm[Mp::REC0 + e] = r1[e];
+    }
+    bool ok = true;
+    for (int t = Nm - 1; t >= 0; --t) {
+        const bool act = t < N;
+        F nxt[PR];
+        __syncwarp();
+        if (act) {
+            if (t >= 1) {
+                const F *rn = scr + Mp::rec(t - 1);
+#pragma unroll
+                for (int r = 0; r < PR; ++r)
+                    if (li + L * r < REC) nxt[r] = rn[li + L * r];
+            }
+            prod_y.run();
+        }
+        __syncwarp();
+        if (act) prod_m.run();
+        __syncwarp();
+        if (act) {
+            // K = -Quu^-1 [Qus | qu] by the 2 x 2 adjugate; Quu not positive definite: K = 0, the
+            // scenario fails
+            const F u00 = sm[Mp::U0], u01 = sm[Mp::U0 + 1], u11 = sm[Mp::U0 + 3];
+            const F det = fma(u00, u11, -(u01 * u01));
+            const bool pd = lq_positive(u00) && lq_positive(det);
+            ok = ok && pd;
+            const F id = pd ? -lq_rcp(det) : F(0);
+#pragma unroll
+            for (int r = 0; r < PK; ++r) {
+                const int e = li + L * r;
+                if (e < KE) {
+                    const bool x1 = e >= NS + 1;
+                    const F own = sm[Mp::H0 + e], other = sm[Mp::H0 + (x1 ? e - (NS + 1) : e + (NS + 1))];
+                    sm[Mp::K0 + e] = fma(x1 ? u00 : u11, own, -(u01 * other)) * id;
+                }
+            }
+        }
+        __syncwarp();
+        if (act) prod_p.run();
+        __syncwarp();
+        if (act) {
+            F *o = scr + Mp::out(N, t);
+#pragma unroll
+            for (int r = 0; r < PO; ++r)
+                if (li + L * r < OUT) o[li + L * r] = sm[om[r]];
+        }
+        __syncwarp();
+        if (act && t >= 1) {
+#pragma unroll
+            for (int r = 0; r < PR; ++r)
+                if (li + L * r < REC) sm[Mp::REC0 + li + L * r] = nxt[r];
+        }
+    }
+    // forward sweep s_{t+1} = F_t s_t + f_t, u_t = K_t s_t + k_t: lane i owns row i of
+    // [F; K] (the controls cost no instruction of their own); the next step's row is
+    // loaded meanwhile
+    __syncwarp();
+    constexpr int NZ = Mp::NZ;
+    static_assert(NZ <= L, "one row of [F; K] per lane");
+    const bool own = live && li < NZ;
+    F x = live && li < NS ? scr[Mp::s0(N) + li] : F(0);
+    constexpr int AHEAD = 4;  // steps: a step takes about 500 cycles, a load from L2 up to 1,500
+    F row[AHEAD][NS], fv[AHEAD];
+    auto fetch = [&](int t, F (&r)[NS], F &f) {
+#pragma unroll
+        for (int k = 0; k < NS; ++k) r[k] = F(0);
+        f = F(0);
+        if (own && t < N) {
+            const F *o = scr + Mp::out(N, t);
+#pragma unroll
+            for (int k = 0; k < NS; ++k) r[k] = o[li * NS + k];
+            f = o[NZ * NS + li];
+        }
+    };
+#pragma unroll
+    for (int d = 0; d < AHEAD; ++d) fetch(d, row[d], fv[d]);
+    bool fin = true;
+    for (int t0 = 0; t0 < Nm; t0 += AHEAD) {
+#pragma unroll
+        for (int d = 0; d < AHEAD; ++d) {
+            const int t = t0 + d;
+            F v = fv[d];
+#pragma unroll
+            for (int k = 0; k < NS; ++k) v = fma(row[d][k], __shfl_sync(0xffffffffu, x, k, L), v);
+            x = v;
+            if (own && t < N) {
+                scr[Mp::sol(N, t) + li] = v;
+                fin = fin && lq_finite(v);
+            }
+            fetch(t + AHEAD, row[d], fv[d]);
+        }
+    }
+    const unsigned bad = __ballot_sync(0xffffffffu, live && !(ok && fin));
+    const unsigned mine = L == 32 ? 0xffffffffu : ((1u << (L & 31)) - 1u) << (g * (L & 31));
+    if (live && li == 0) a.ok[s] = (bad & mine) == 0u;
+    }
+}
+
+// s, u from the sweep, then the box block and the poses of the new iterate
+template <typename T, typename F, int KIND>
+__global__ void __launch_bounds__(kTrajBlock) k_traj_apply(RicArgs<T> a, const int *lq_ok) {
+    constexpr int NS = MDims<KIND>::NS, NU = MDims<KIND>::NU, NZ = NS + NU;
+    using Mp = RicMap<KIND>;
+    const int s = blockIdx.x, lane = threadIdx.x, NT = blockDim.x;
+    if (a.scen_status[s] != kActive) return;
+    const ScenMeta sm = a.meta[s];
+    const int N = sm.N;
+    const F *scr = reinterpret_cast<const F *>(a.scratch) + a.scratch0[s];
+    const bool ok = lq_ok[s] != 0;
+    double rpb = 0.0, rdb = 0.0;
+    for (int t = lane; t < N; t += NT) {
+        const F *sol = scr + Mp::sol(N, t);
+        F v[NZ];
+        T st[NS], ut[NU];
+#pragma unroll
+        for (int i = 0; i < NZ; ++i) v[i] = sol[i];
+#pragma unroll
+        for (int i = 0; i < NS; ++i) a.s[(long long)(sm.state0 + t + 1) * NS + i] = st[i] = T(v[i]);
+#pragma unroll
+        for (int i = 0; i < NU; ++i) a.u[(long long)(sm.ctrl0 + t) * NU + i] = ut[i] = T(v[NS + i]);
+        if (ok) box_poses<T, KIND>(a, sm, t, st, ut, rpb, rdb);
+    }
+    if (!ok) {
+        // k_traj_lq has advanced the counter: iteration j is *iter - 1
+        __syncthreads();
+        if (lane < 32) finish_scenario<T, KIND>(a, sm, s, OCA_SCEN_FAILED, *a.iter - 1, 0.0, 0.0);
+        return;
+    }
+    __shared__ double part[kTrajBlock / 32][2];
+    rpb = warp_sum(rpb);
+    rdb = warp_sum(rdb);
+    if ((lane & 31) == 0) {
+        part[lane >> 5][0] = rpb;
+        part[lane >> 5][1] = rdb;
+    }
+    __syncthreads();
+    if (lane == 0) {
+        for (int w = 1; w < NT / 32; ++w) {
+            rpb += part[w][0];
+            rdb += part[w][1];
+        }
+        a.box_res[2 * s] = rpb;
+        a.box_res[2 * s + 1] = rdb;
+    }
+}
+
+// Lanes per scenario: a warp of the recursion issues 22 (L = 32) or 24 (L = 16)
+// FP64 instructions per stage, so 16 lanes carry nearly twice the scenarios; with
+// no more scenarios than schedulers (4 per SM) every one has its own warp and 32
+// lanes are the shorter chain (256 scenarios of horizon 50: 2,290 cycles per stage).
+// 2,048 scenarios: 138 us with 16 lanes, 174 with 32.
+template <typename T, typename F, int KIND>
+cudaError_t launch_traj(const RicArgs<T> &a, int *lq_ok, const int *order, int max_n, int n_sm, cudaStream_t st) {
+    LqArgs2<F> l;
+    l.meta = a.meta;
+    l.order = order;
+    l.n_scen = a.n_scen;
+    l.scen_status = a.scen_status;
+    l.scratch = a.scratch;
+    l.scratch0 = a.scratch0;
+    l.dt = F(a.model.dt);
+    for (int i = 0; i < 2; ++i)
+        l.ru[i] = F(2) * F(a.model.Qu[i]) + F(a.damp) +
+                  (a.model.u_lo[i] > T(-1e29) || a.model.u_hi[i] < T(1e29) ? F(a.rho_box) : F(0));
+    l.ok = lq_ok;
+    l.iter = a.iter;
+    const int steps = std::min(kTrajBlock, (max_n + 1 + 31) / 32 * 32);
+    k_traj_stage<T, F, KIND><<<a.n_scen, steps, sizeof(F) * steps * traj_rec_stride<F, KIND>(), st>>>(a);
+    const int one = a.n_scen <= 4 * n_sm, groups = one ? a.n_scen : (a.n_scen + 1) / 2, ctas = std::min(n_sm, groups);
+    if (one) k_traj_lq<F, KIND, 32><<<ctas, 32 * kLqWarps, 0, st>>>(l);
+    else k_traj_lq<F, KIND, 16><<<ctas, 32 * kLqWarps, 0, st>>>(l);
+    k_traj_apply<T, F, KIND><<<a.n_scen, steps, 0, st>>>(a, lq_ok);
     return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_riccati(const RicArgs<T> &a, bool f32, cudaStream_t st) {
-    if (f32) return launch_riccati_f<T, float>(a, st);
-    return launch_riccati_f<T, double>(a, st);
+template <typename T, typename F>
+cudaError_t launch_riccati_f(const RicArgs<T> &a, int *lq_ok, const int *order, int max_n, int n_sm, cudaStream_t st) {
+    switch (a.model.kind) {
+        case 0: return launch_traj<T, F, 0>(a, lq_ok, order, max_n, n_sm, st);
+        case 1: return launch_traj<T, F, 1>(a, lq_ok, order, max_n, n_sm, st);
+        case 2: {
+            k_riccati<T, F, 2, 128><<<a.n_scen, 128, 0, st>>>(a);
+            k_advance<<<1, 1, 0, st>>>(a.iter);
+            return cudaGetLastError();
+        }
+    }
+    return cudaErrorInvalidValue;
 }
 
-template cudaError_t launch_riccati<float>(const RicArgs<float> &, bool, cudaStream_t);
-template cudaError_t launch_riccati<double>(const RicArgs<double> &, bool, cudaStream_t);
+template <typename T>
+cudaError_t launch_riccati(const RicArgs<T> &a, bool f32, int *lq_ok, const int *order, int max_n, int n_sm, cudaStream_t st) {
+    if (f32) return launch_riccati_f<T, float>(a, lq_ok, order, max_n, n_sm, st);
+    return launch_riccati_f<T, double>(a, lq_ok, order, max_n, n_sm, st);
+}
+
+template cudaError_t launch_riccati<float>(const RicArgs<float> &, bool, int *, const int *, int, int, cudaStream_t);
+template cudaError_t launch_riccati<double>(const RicArgs<double> &, bool, int *, const int *, int, int, cudaStream_t);
 
 }  // namespace oca
