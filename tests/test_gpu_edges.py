@@ -1,0 +1,85 @@
+"""Kernels on a scene whose tiles mix what the benchmark's scenes keep apart: five
+parts of 3 to 8 faces per scenario (so that neighbouring lanes sit on parts with
+different face counts), horizons from 1, one to 17 obstacles of 3 to 24 faces."""
+import math
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2406_07048_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2406_07048_gb300 import _build, binding
+    _build.build()
+    return binding
+
+
+def _ngon(k, r, off):
+    ang = 2.0 * math.pi * np.arange(k) / k + 0.1
+    return np.stack([np.cos(ang), np.sin(ang)], 1), np.full(k, r), 0, np.array([off, 0.0])
+
+
+def _mixed(dtype):
+    model = synth.bicycle_model()
+    scens = []
+    for s, (N, M) in enumerate([(1, 1), (2, 9), (5, 17), (13, 3), (40, 8)]):
+        rng = np.random.default_rng([31, s])
+        obs = []
+        for j in range(M):
+            C, off = synth.random_polygon(rng, [3, 24, 7, 12][j % 4], 0.5, 2.0)
+            obs.append((C, off, np.array([rng.uniform(5.0, 40.0), rng.uniform(0.0, 10.0)])))
+        parts = [_ngon(k, 0.5 + 0.1 * k, 0.3 * k) for k in (3, 8, 4, 5, 6)]
+        scens.append(synth._Scen(obs, parts, N, synth._ref_2d(model, N, 0.0, 2.0 * N, 5.0), np.zeros((N, model.nu))))
+    sc = synth._assemble(model, scens, "mixed-parts")
+    if dtype == torch.float32:  # the geometry as the library stores it
+        for f in ("obs_C", "obs_d", "part_A", "part_b", "part_off", "s_ref", "s_init"):
+            setattr(sc, f, getattr(sc, f).astype(np.float32).astype(np.float64))
+    return sc
+
+
+def _rounded(a, dtype):
+    return a.astype(np.float32).astype(np.float64) if dtype == torch.float32 else a
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("warps", [1, 5])
+def test_cert_margin_mixed_parts(B, ora, dtype, warps):
+    """Margins of random sparse duals (with a negative, an infinite and a NaN one)
+    against the oracle's FP64 bound on the same stored numbers: sums of at most 32
+    products in another order (1e-12, floored at 1)."""
+    sc = _mixed(dtype)
+    rng = np.random.default_rng(5)
+    states = _rounded(synth.random_states(sc, rng, 1.0, 0.4), dtype)
+    P = sc.n_pairs
+    lam = _rounded(rng.exponential(1.0, (P, sc.fr_max)) * (rng.uniform(size=(P, sc.fr_max)) < 0.5), dtype)
+    mu = _rounded(rng.exponential(1.0, (P, sc.fo_max)) * (rng.uniform(size=(P, sc.fo_max)) < 0.2), dtype)
+    bad = {3: -1.0, 40: np.inf, 77: np.nan}
+    for p, v in bad.items():
+        mu[p, 0] = v
+    ds = B.DeviceScene(B.Context(0), sc, dtype)
+    ds.warps = warps
+    m_g = B.cert_margin(ds, ds.tensor(states), ds.to_device_pairs(lam), ds.to_device_pairs(mu)).cpu().numpy()
+    pb, sb = sc.pair_begin, sc.state_begin
+    for p in range(P):
+        if p in bad:
+            assert m_g[p] < -1e300
+            continue
+        s = int(np.searchsorted(pb, p, side="right")) - 1
+        N, NP, l = int(sc.horizon[s]), sc.n_parts(s), p - int(pb[s])
+        gm, gp, t = int(sc.obs_begin[s]) + l // (N * NP), int(sc.part_begin[s]) + l // N % NP, l % N + 1
+        nr, nf = int(sc.part_nf[gp]), int(sc.obs_nf[gm])
+        rho, R = ora.part_pose(sc.model, 0, sc.part_off[gp], states[int(sb[s]) + t])[:2]
+        Cb, db = sc.obs_C[gm, :nf] @ R, sc.obs_d[gm, :nf] - sc.obs_C[gm, :nf] @ rho
+        want = ora.cert_margin(sc.part_A[gp, :nr], sc.part_b[gp, :nr], Cb, db, lam[p, :nr], mu[p, :nf])
+        if not np.isfinite(want):
+            assert m_g[p] < -1e300
+        else:
+            assert abs(m_g[p] - want) <= 1e-12 * max(1.0, abs(want)), (p, m_g[p], want)
