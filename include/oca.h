@@ -144,8 +144,9 @@ oca_status oca_scene_info_get(const oca_scene *scene, oca_scene_info *info);
 
 /* Work shape of the pair kernels: warps per 32-lane tile (1..16); each warp
  * sweeps every W-th obstacle of the tile's scenario.  oca_scene_create picks
- * about eight obstacles per warp at the median obstacle count;
- * DeviceScene.autotune_warps in the Python binding times the fused pair
+ * it from the number of tiles (few tiles: up to one warp per obstacle, many:
+ * two), and another for the LP and margin kernels; a count set here holds for
+ * all of them.  DeviceScene.autotune_warps in the Python binding times the fused pair
  * kernel of short solves for each candidate and sets the fastest.
  * Errors: OCA_ERR_INVALID_ARGUMENT (warps outside 1..16), OCA_ERR_CAPACITY
  * (more warps per tile than the pair kernels are compiled for -- 16 for

@@ -30,7 +30,8 @@ struct oca_scene {
     std::vector<ScenMeta> meta;
     std::vector<int64_t> pair_begin, state_begin, ctrl_begin;
     int64_t P = 0, n_states = 0, n_ctrls = 0;
-    int Qtot = 0, maxQ = 0, n_tiles = 0, ny_max = 0, W = 1, maxN = 0, maxM = 0;
+    int Qtot = 0, maxQ = 0, n_tiles = 0, ny_max = 0, maxN = 0, maxM = 0;
+    int W = 1, W_lp = 1;  // warps per tile: pair kernels, LP and margin kernels
     const void *obs_C = nullptr, *obs_d = nullptr, *part_A = nullptr, *part_b = nullptr, *part_off = nullptr;
     // device
     ScenMeta *d_meta = nullptr;
@@ -286,7 +287,7 @@ oca_status scale_impl(oca_scene *sc, const oca_model *m, const void *states, voi
     a.margin = margin;
     a.verdict = verdict;
     a.status = status;
-    OCA_CK(launch_scale<T>(a, sc->dim, sc->n_tiles, sc->W, st));
+    OCA_CK(launch_scale<T>(a, sc->dim, sc->n_tiles, sc->W_lp, st));
     return OCA_OK;
 }
 
@@ -304,7 +305,7 @@ oca_status cert_impl(oca_scene *sc, const oca_model *m, const void *states, cons
     a.lambda = static_cast<const T *>(lambda);
     a.mu = static_cast<const T *>(mu);
     a.margin = margin;
-    OCA_CK(launch_cert<T>(a, sc->n_tiles, sc->W, st));
+    OCA_CK(launch_cert<T>(a, sc->n_tiles, sc->W_lp, st));
     return OCA_OK;
 }
 
@@ -1034,7 +1035,6 @@ oca_status oca_scene_create(oca_ctx *ctx, const oca_scene_desc *d, oca_scene **o
     sc->ctrl_begin.assign(S + 1, 0);
     long long qtot = 0, tiles = 0;
     std::vector<long long> cost(S);
-    std::vector<int> Ms;
     for (int s = 0; s < S; ++s) {
         ScenMeta &m = sc->meta[s];
         m.N = d->horizon[s];
@@ -1060,7 +1060,6 @@ oca_status oca_scene_create(oca_ctx *ctx, const oca_scene_desc *d, oca_scene **o
         long long faces = 0;
         for (int j = 0; j < m.M; ++j) faces += d->obs_nf[m.obs0 + j] + 1;
         cost[s] = faces;
-        Ms.push_back(m.M);
     }
     if (qtot > (1LL << 30) || tiles > (1LL << 30) || sc->state_begin[S] > (1LL << 30)) {
         free_scene(sc);
@@ -1086,11 +1085,25 @@ oca_status oca_scene_create(oca_ctx *ctx, const oca_scene_desc *d, oca_scene **o
     std::vector<int> by_horizon(S);
     for (int s = 0; s < S; ++s) by_horizon[s] = s;
     std::stable_sort(by_horizon.begin(), by_horizon.end(), [&](int x, int y) { return sc->meta[x].N > sc->meta[y].N; });
-    // warps per tile: about 8 obstacles per warp at the median obstacle count
-    std::nth_element(Ms.begin(), Ms.begin() + Ms.size() / 2, Ms.end());
-    const int Mmed = Ms[Ms.size() / 2];
-    sc->W = std::max(1, std::min(16, (Mmed + 7) / 8));
+    // Warps per tile (until oca_scene_set_warps): as many as keep the launch within
+    // 2.5 times the warps that an SM holds (16, 12 in FP64 and 8 in 3-D of the pair
+    // kernel, 32 of the LP and margin kernels, by their registers), a power of two so
+    // that whole CTAs fill them, no more than obstacles.  Few tiles then spread their
+    // obstacles over idle SMs, many tiles amortise a warp's set-up over more of them.
+    // Pair kernel, us per launch: 5,660 trailer tiles 706 with 2 (773 with 5), 1,470
+    // tiles 208 with 4 (251 with 2, 226 with 8), 345 tiles 74 with 16 (98 with 5), one
+    // tile of 4 obstacles in FP64 91 with 4 (264 with 1); LP kernel: 2,892 tiles 1,306
+    // with 4 (1,468 with 2), 4 tiles 100 with 16 (239 with 4); margin kernel: 5,660 tiles
+    // 1,107 with 4 (1,134 with 2).
+    auto pick = [&](int per_sm, int most, int least) {
+        int w = 16;
+        while (w > 1 && (w > most || (w > least && (double)tiles * w > 2.5 * per_sm * ctx->n_sm))) w /= 2;
+        return std::max(1, std::min(w, sc->maxM));
+    };
+    const int pair_warps = pair_max_warps(d->dim, dsize(d->dtype));
+    sc->W = pick(pair_warps, pair_warps, 2);
     while (sc->W > 1 && !warps_fit(sc, sc->W)) --sc->W;
+    sc->W_lp = pick(32, 16, 4);
 
     const size_t ts = dsize(d->dtype);
     const int PK = d->dim + d->dim * d->dim;
@@ -1191,7 +1204,7 @@ oca_status oca_scene_info_get(const oca_scene *sc, oca_scene_info *info) {
 oca_status oca_scene_set_warps(oca_scene *sc, int warps) {
     if (!sc || warps < 1 || warps > 16) return OCA_ERR_INVALID_ARGUMENT;
     if (!warps_fit(sc, warps)) return OCA_ERR_CAPACITY;
-    sc->W = warps;
+    sc->W = sc->W_lp = warps;
     return OCA_OK;
 }
 
