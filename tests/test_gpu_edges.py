@@ -83,3 +83,24 @@ def test_cert_margin_mixed_parts(B, ora, dtype, warps):
             assert m_g[p] < -1e300
         else:
             assert abs(m_g[p] - want) <= 1e-12 * max(1.0, abs(want)), (p, m_g[p], want)
+
+
+@pytest.mark.parametrize("ns,nu,N,S", [(2, 1, 63, 3), (5, 2, 64, 1), (12, 4, 65, 3), (7, 3, 71, 2), (6, 4, 520, 1), (4, 2, 72, 40)])
+@pytest.mark.parametrize("method", [0, 1])
+def test_lq_chunked_rollout_edges(B, ora, ns, nu, N, S, method):
+    """Horizons around the chunked rollout's start and its remainders, unrolled and
+    run-time dimensions, against the oracle's textbook recursion (1e-9 relative)."""
+    from tests.test_oracle_riccati import _rand_lq
+    rng = np.random.default_rng(100 * ns + N)
+    probs = [_rand_lq(rng, N, ns, nu) for _ in range(S)]
+    for pr in probs:
+        pr[0][:] *= 0.9  # the closed loop stays bounded over the longer horizons
+    dev = [torch.as_tensor(np.stack([pr[i] for pr in probs]), dtype=torch.float64, device="cuda") for i in range(8)]
+    out = B.lq_solve(B.Context(0), *dev, method=method)
+    torch.cuda.synchronize()
+    assert (out["status"].cpu().numpy() == 0).all()
+    for k in {0, S // 2, S - 1}:
+        s_o, u_o, st = ora.riccati(*probs[k])
+        assert st == 0
+        for got, want in ((out["s"][k], s_o), (out["u"][k], u_o)):
+            assert np.abs(got.cpu().numpy() - want).max() <= 1e-9 * max(1.0, np.abs(want).max())
