@@ -104,3 +104,11 @@ def test_lq_chunked_rollout_edges(B, ora, ns, nu, N, S, method):
         assert st == 0
         for got, want in ((out["s"][k], s_o), (out["u"][k], u_o)):
             assert np.abs(got.cpu().numpy() - want).max() <= 1e-9 * max(1.0, np.abs(want).max())
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+def test_cold_start_on_the_device(B, dtype):
+    """The device's cold start is the scene's, element for element."""
+    for sc in (_mixed(dtype), synth.config3(n_scen=5), synth.config4(n_scen=2, n_obs=8, N=5), synth.config_max()):
+        ds = B.DeviceScene(B.Context(0), sc, dtype)
+        assert torch.equal(ds.cold_y(), ds.to_device_pairs(sc.cold_y()))
