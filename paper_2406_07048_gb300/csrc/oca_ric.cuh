@@ -362,14 +362,8 @@ __device__ __forceinline__ bool spd_inverse(const F (&U)[NU][NU], F (&X)[NU][NU]
     }
 }
 
-template <int NT>
-__device__ __forceinline__ void ric_sync() {
-    if constexpr (NT == 32) __syncwarp();
-    else __syncthreads();
-}
-
-// NT threads (one warp, or the whole CTA when NT > 32) run the recursion
-template <typename F, int NS, int NU, int NT = 32>
+// one warp runs the recursion
+template <typename F, int NS, int NU>
 __device__ bool ric_factor(F *scr, int N, const F *ru_diag) {
     using LY = RicLayout<NS, NU>;
     constexpr int NX = NS + NU + 1;           // columns of G = [A | B | c]
@@ -377,10 +371,11 @@ __device__ bool ric_factor(F *scr, int N, const F *ru_diag) {
     constexpr int MC = NZ + 1;                // columns of M as stored
     constexpr int NG = NS * NX, NQ = NS * NS;
     constexpr int NST = NG + NQ + NS + NU;    // staged values per step
+    constexpr int NT = 32;
     constexpr int PF = (NST + NT - 1) / NT;   // of them per thread
     constexpr int NSYM = NZ * (NZ + 1) / 2;   // upper triangle of the Hessian part of M
     constexpr int NPS = NS * (NS + 1) / 2;    // upper triangle of P
-    const int lane = threadIdx.x;  // thread of the NT
+    const int lane = threadIdx.x;
     __shared__ F P[NS * NS], pv[NS], stg[NST], Y[NS * NX], M[NZ * MC], KK[NU * (NS + 1)];
     const F *Gs = stg, *Qs = stg + NG, *qs = stg + NG + NQ, *rs = stg + NG + NQ + NS;
     for (int e = lane; e < NS * NS; e += NT) P[e] = scr[LY::Q(N, N) + e];
@@ -393,50 +388,6 @@ __device__ bool ric_factor(F *scr, int N, const F *ru_diag) {
             if (e < NST) nxt[r] = ric_stage_elem<F, NS, NU>(scr, N, N - 1, e);
         }
     }
-    // each thread's entries of the stage matrix M (upper triangle row by row,
-    // then the gradient column) and of P (upper triangle, then p): their (i, j)
-    // depend on the thread only.  With NT > 32 (the 12-state model: 152 and 90
-    // entries per step) they are found once, before the steps; a one-warp group
-    // (27-35 entries) finds them in each step, which measured faster there.
-    constexpr bool HOIST = NT > 32;
-    constexpr int RM = HOIST ? (NSYM + NZ + NT - 1) / NT : 1, RP = HOIST ? (NPS + NS + NT - 1) / NT : 1;
-    int mi[RM], mj[RM], pi_[RP], pj[RP];
-    if constexpr (HOIST) {
-#pragma unroll
-        for (int r = 0; r < RM; ++r) {
-            const int e = lane + NT * r;
-            int i = 0, j = NZ;
-            if (e < NSYM) {
-                int rem = e;
-                while (rem >= NZ - i) {
-                    rem -= NZ - i;
-                    ++i;
-                }
-                j = i + rem;
-            } else {
-                i = e - NSYM;
-            }
-            mi[r] = i;
-            mj[r] = j;
-        }
-#pragma unroll
-        for (int r = 0; r < RP; ++r) {
-            const int e = lane + NT * r;
-            int i = 0, j = NS;  // j = NS marks p_i
-            if (e < NPS) {
-                int rem = e;
-                while (rem >= NS - i) {
-                    rem -= NS - i;
-                    ++i;
-                }
-                j = i + rem;
-            } else {
-                i = e - NPS;
-            }
-            pi_[r] = i;
-            pj[r] = j;
-        }
-    }
     bool ok = true;
     for (int t = N - 1; t >= 0; --t) {
 #pragma unroll
@@ -444,7 +395,7 @@ __device__ bool ric_factor(F *scr, int N, const F *ru_diag) {
             const int e = lane + NT * r;
             if (e < NST) stg[e] = nxt[r];
         }
-        ric_sync<NT>();
+        __syncwarp();
         if (t >= 1) {
 #pragma unroll
             for (int r = 0; r < PF; ++r) {
@@ -460,24 +411,8 @@ __device__ bool ric_factor(F *scr, int N, const F *ru_diag) {
             for (int l = 0; l < NS; ++l) acc += P[k * NS + l] * Gs[l * NX + j];
             Y[e] = acc;
         }
-        ric_sync<NT>();
+        __syncwarp();
         // M: the upper triangle of the Hessian part, then the gradient column
-        if constexpr (HOIST) {
-#pragma unroll
-            for (int r = 0; r < RM; ++r) {
-                if (lane + NT * r >= NSYM + NZ) break;
-                const int i = mi[r], j = mj[r];
-                const int jy = j < NZ ? j : NX - 1;
-                F acc;
-                if (j == NZ) acc = i < NS ? qs[i] : rs[i - NS];
-                else if (j < NS) acc = Qs[i * NS + j];
-                else acc = (i == j) ? ru_diag[i - NS] : F(0);
-#pragma unroll
-                for (int k = 0; k < NS; ++k) acc += Gs[k * NX + i] * Y[k * NX + jy];
-                M[i * MC + j] = acc;
-                if (j < NZ && j != i) M[j * MC + i] = acc;
-            }
-        } else
         for (int e = lane; e < NSYM + NZ; e += NT) {
             int i, j;
             if (e < NSYM) {
@@ -502,7 +437,7 @@ __device__ bool ric_factor(F *scr, int N, const F *ru_diag) {
             M[i * MC + j] = acc;
             if (j < NZ && j != i) M[j * MC + i] = acc;
         }
-        ric_sync<NT>();
+        __syncwarp();
         // Quu^-1 (every lane), then [K_t | k_t] = -Quu^-1 [Qus | qu]
         F U[NU][NU], X[NU][NU];
 #pragma unroll
@@ -520,27 +455,8 @@ __device__ bool ric_factor(F *scr, int N, const F *ru_diag) {
             if (j < NS) scr[LY::K(N, t) + a * NS + j] = acc;
             else scr[LY::k(N, t) + a] = acc;
         }
-        ric_sync<NT>();
+        __syncwarp();
         // P_t = Qss + Qus^T K_t (upper triangle, mirrored), p_t = qs + Qus^T k_t
-        if constexpr (HOIST) {
-#pragma unroll
-            for (int r = 0; r < RP; ++r) {
-                if (lane + NT * r >= NPS + NS) break;
-                const int i = pi_[r], j = pj[r];
-                if (j < NS) {
-                    F acc = M[i * MC + j];
-#pragma unroll
-                    for (int a = 0; a < NU; ++a) acc += M[(NS + a) * MC + i] * KK[a * (NS + 1) + j];
-                    P[i * NS + j] = acc;
-                    P[j * NS + i] = acc;
-                } else {
-                    F acc = M[i * MC + NZ];
-#pragma unroll
-                    for (int a = 0; a < NU; ++a) acc += M[(NS + a) * MC + i] * KK[a * (NS + 1) + NS];
-                    pv[i] = acc;
-                }
-            }
-        } else
         for (int e = lane; e < NPS + NS; e += NT) {
             if (e < NPS) {
                 int rem = e, i = 0;
@@ -562,10 +478,9 @@ __device__ bool ric_factor(F *scr, int N, const F *ru_diag) {
                 pv[i] = acc;
             }
         }
-        ric_sync<NT>();
+        __syncwarp();
     }
-    if constexpr (NT == 32) return __all_sync(0xffffffffu, ok);
-    else return __syncthreads_and(ok) != 0;
+    return __all_sync(0xffffffffu, ok);
 }
 
 // Forward sweep u_t = K_t s_t + k_t, s_{t+1} = A_t s_t + B_t u_t + c_t from

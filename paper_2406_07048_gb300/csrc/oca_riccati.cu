@@ -16,8 +16,6 @@
 //      per-(part, t) statistics W, Wc, E through the pose Jacobians;
 //   3. runs the backward Riccati recursion (factorisation precision F) and
 //      the forward sweep, writing s^{j+1}, u^{j+1} and the new poses.
-// The 2-D models run as three kernels (below), the 12-state model as one kernel
-// with a four-warp CTA per scenario.
 #include <algorithm>
 #include <type_traits>
 
@@ -33,7 +31,7 @@ long long riccati_scratch_elems(int kind, int N) {
         // the forward step's packed records and the adjoint's dense layout share the block
         case 0: return std::max(RicLayout<4, 2>::size(N), RicMap<0>::size(N));
         case 1: return std::max(RicLayout<5, 2>::size(N), RicMap<1>::size(N));
-        default: return RicLayout<12, 4>::size(N);
+        default: return std::max(RicLayout<12, 4>::size(N), RicMap<2>::size(N));
     }
 }
 
@@ -164,128 +162,13 @@ __device__ __forceinline__ void box_poses(const RicArgs<T> &a, const ScenMeta &s
         if (bu[i]) update(ut[i], a.model.u_lo[i], a.model.u_hi[i], zu[i], wu[i], a.box_zu + ku + i, a.box_wu + ku + i);
 }
 
-__global__ void k_advance(int *iter) { *iter += 1; }
-
-// NT threads per scenario: warp 0 runs every phase but the Riccati
-// recursion, which all NT threads share (NT > 32 for the 12-state model,
-// whose per-step products have 150-200 entries).
-template <typename T, typename F, int KIND, int NT>
-__global__ void __launch_bounds__(NT) k_riccati(RicArgs<T> a) {
-    constexpr int NS = MDims<KIND>::NS, NU = MDims<KIND>::NU, D = MDims<KIND>::D;
-    const int s = blockIdx.x;
-    const int lane = threadIdx.x;
-    if (a.scen_status[s] != kActive) return;
-    const int j = *a.iter;
-    if (j > a.max_iter) return;
-    const ScenMeta sm = a.meta[s];
-    const int N = sm.N;
-    __shared__ int s_retired;
-
-    // ---- 1. stopping rule of iteration j-1 (warp 0)
-    if (lane < 32) {
-        const bool r = stop_rule<T, KIND>(a, sm, s, j);
-        if (lane == 0) s_retired = r;
-    }
-    ric_sync<NT>();
-    if (s_retired) return;
-
-    F *scr = reinterpret_cast<F *>(a.scratch) + a.scratch0[s];
-
-    // ---- 2. stage assembly, lanes over t (in the array precision T; only
-    // the factorisation below runs in F)
-    StageParams<T> sp;
-    StageSrc<T> src;
-    stage_inputs(a, sp, src);
-    for (int t = lane; t <= N; t += NT) assemble_stage<T, F, KIND>(sp, src, sm, t, scr);
-    ric_sync<NT>();
-
-    // ---- 3. backward Riccati recursion (all NT threads), 4. forward sweep (warp 0)
-    // diagonal of Ru, formed once and shared by the NT threads (a per-thread
-    // copy indexed at run time gave wrong values in threads >= 32 of the
-    // FP64 four-warp instantiation; the shared copy is also less work)
-    __shared__ F ru_diag[NU];
-    for (int i = lane; i < NU; i += NT)
-        ru_diag[i] = F(2) * F(a.model.Qu[i]) + F(a.damp) +
-                     (bounded(a.model.u_lo[i], a.model.u_hi[i]) ? F(a.rho_box) : F(0));
-    ric_sync<NT>();
-    bool ok = ric_factor<F, NS, NU, NT>(scr, N, ru_diag);
-    if (lane >= 32) return;
-    __shared__ F sc[NS];
-    for (int i = lane; i < NS; i += 32) sc[i] = F(a.s[(long long)sm.state0 * NS + i]);
-    __syncwarp();
-    struct Out {
-        T *s, *u;
-        long long s0, c0;
-        __device__ void put_u(int t, int i, F v) { u[(c0 + t) * NU + i] = T(v); }
-        __device__ void put_s(int t, int i, F v) { s[(s0 + t) * NS + i] = T(v); }
-    } out{a.s, a.u, (long long)sm.state0, (long long)sm.ctrl0};
-    ok = ric_sweep<F, NS, NU>(scr, N, sc, out) && ok;
-    if (!ok) {
-        finish_scenario<T, KIND>(a, sm, s, OCA_SCEN_FAILED, j, 0.0, 0.0);
-        return;
-    }
-    __syncwarp();
-    // ---- box block: z = clip((s,u)^{j+1} + w), w += (s,u)^{j+1} - z
-    double rpb = 0.0, rdb = 0.0;
-    const int n_box = a.rho_box > T(0) ? N * NS + N * NU : 0;  // rho_box = 0: no box block
-    for (int e = lane; e < n_box; e += 32) {
-        long long k2;
-        T lo, hi, x;
-        T *zz, *ww;
-        if (e < N * NS) {
-            const int t = 1 + e / NS, i = e % NS;
-            lo = a.model.s_lo[i];
-            hi = a.model.s_hi[i];
-            k2 = (long long)(sm.state0 + t) * NS + i;
-            x = a.s[k2];
-            zz = a.box_zs;
-            ww = a.box_ws;
-        } else {
-            const int e2 = e - N * NS, t = e2 / NU, i = e2 % NU;
-            lo = a.model.u_lo[i];
-            hi = a.model.u_hi[i];
-            k2 = (long long)(sm.ctrl0 + t) * NU + i;
-            x = a.u[k2];
-            zz = a.box_zu;
-            ww = a.box_wu;
-        }
-        if (!bounded(lo, hi)) continue;
-        const T zn = fmin(fmax(x + ww[k2], lo), hi);
-        rdb += double(zn - zz[k2]) * double(zn - zz[k2]);
-        rpb += double(x - zn) * double(x - zn);
-        zz[k2] = zn;
-        ww[k2] += x - zn;
-    }
-    rpb = warp_sum(rpb);
-    rdb = warp_sum(rdb);
-    if (lane == 0) {
-        a.box_res[2 * s] = rpb;
-        a.box_res[2 * s + 1] = rdb;
-    }
-    // ---- poses of s^{j+1} for the next pair kernel
-    const int Q = sm.NP * N;
-    for (int q = lane; q < Q; q += 32) {
-        const int part = q / N, t = q % N + 1;
-        const int gp = sm.part0 + part;
-        T st[NS], off[D], rho[D], R[D * D];
-        for (int i = 0; i < NS; ++i) st[i] = a.s[(long long)(sm.state0 + t) * NS + i];
-#pragma unroll
-        for (int i = 0; i < D; ++i) off[i] = a.g.part_off[gp * D + i];
-        part_pose<T, KIND>(a.model, a.g.part_link[gp], off, st, rho, R, nullptr, nullptr, nullptr);
-        const int col = sm.qbeg + q;
-#pragma unroll
-        for (int i = 0; i < D; ++i) a.pose[(long long)i * a.Qtot + col] = rho[i];
-#pragma unroll
-        for (int i = 0; i < D * D; ++i) a.pose[(long long)(D + i) * a.Qtot + col] = R[i];
-    }
-}
-
 // ============================================================================
-// 2-D models: three kernels per trajectory step.
+// Three kernels per trajectory step.
 //   k_traj_stage   stopping rule and stage assembly, lanes over t (FP32 work with
 //                  everything in registers, written as one packed record per stage)
-//   k_traj_lq      backward recursion and forward sweep (the FP64 chain), L lanes
-//                  per scenario, 32 / L scenarios per warp
+//   k_traj_lq      backward recursion and forward sweep (the FP64 chain): 2-D models,
+//                  L lanes per scenario, 32 / L scenarios per warp
+//   k_traj_lq4     the same for the 12-state model, four warps per scenario
 //   k_traj_apply   the new iterate in T, box block and poses, lanes over t
 // The recursion is bound by FP64 issue (oca_ricprog.cuh), the other two by latency;
 // apart, the recursion keeps one warp per scheduler busy with nothing but the
@@ -384,8 +267,232 @@ struct LqSlotsOf<F, RicPhase<SLOTS, L>> {
 
 // threads per scenario of the per-step kernels: one per horizon step up to 96
 constexpr int kTrajBlock = 96;
+// shared elements per thread of k_traj_stage (the 12-state record is written directly)
 template <typename F, int KIND>
-constexpr int traj_rec_stride() { return RicMap<KIND>::REC | 1; }
+constexpr int traj_rec_stride() { return KIND == 2 ? 0 : RicMap<KIND>::REC | 1; }
+
+// Stage t of the 12-state model as a packed record, in T: only the entries of A and B
+// that are not structurally 0 or 1, and the Gauss-Newton terms of the six coordinates
+// (position, angles) that a part's pose depends on.  (The generic assembly over dense
+// 12 x 12 arrays keeps 2 KB per thread in local memory.)
+template <typename T, typename F>
+__device__ void quad_record(const StageParams<T> &a, const StageSrc<T> &src, const ScenMeta &sm, int t, F *rec) {
+    using Mp = RicMap<2>;
+    constexpr int NS = 12, NU = 4;
+    const DevModel<T> &m = a.model;
+    const int N = sm.N;
+    T st[NS];
+    const long long ks = (long long)(sm.state0 + t) * NS;
+#pragma unroll
+    for (int i = 0; i < NS; ++i) st[i] = src.s[ks + i];
+    T R[9], dR[3][9];
+    rot3<T>(st[6], st[7], st[8], R, dR);
+    if (t < N) {
+        T ut[NU];
+        const long long ku = (long long)(sm.ctrl0 + t) * NU;
+#pragma unroll
+        for (int i = 0; i < NU; ++i) ut[i] = src.u[ku + i];
+        T f[NS];
+        dynamics<T, 2>(m, st, ut, f, nullptr, nullptr);
+        const T mass = m.p[0], Jx = m.p[2], Jy = m.p[3], Jz = m.p[4], arm = m.p[5], km = m.p[6], dt = m.dt;
+        const T thrust = mass * m.p[1] + ut[0] + ut[1] + ut[2] + ut[3];
+        const T p = st[9], q = st[10], r = st[11];
+        const T cf = m_cos(st[6]), sf = m_sin(st[6]), ct = m_cos(st[7]), tt = m_tan(st[7]), sc = T(1) / ct;
+        const T w1 = sf * q + cf * r, w2 = cf * q - sf * r;
+        // df/ds and df/du in the order of RicSparse<2>
+        T A[25], B[9];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                if (i < 2 || k < 2) A[i * 3 + k] = dt * (dR[k][i * 3 + 2] * thrust / mass);
+            B[i] = dt * (R[i * 3 + 2] / mass);
+        }
+        A[8] = T(1) + dt * (w2 * tt);
+        A[9] = dt * (w1 * sc * sc);
+        A[10] = dt * (sf * tt);
+        A[11] = dt * (cf * tt);
+        A[12] = dt * -w1;
+        A[13] = dt * cf;
+        A[14] = dt * -sf;
+        A[15] = dt * (w2 * sc);
+        A[16] = dt * (w1 * sc * tt);
+        A[17] = dt * (sf * sc);
+        A[18] = dt * (cf * sc);
+        A[19] = dt * (r * (Jy - Jz) / Jx);
+        A[20] = dt * (q * (Jy - Jz) / Jx);
+        A[21] = dt * (r * (Jz - Jx) / Jy);
+        A[22] = dt * (p * (Jz - Jx) / Jy);
+        A[23] = dt * (q * (Jx - Jy) / Jz);
+        A[24] = dt * (p * (Jx - Jy) / Jz);
+        B[3] = dt * (arm / Jx);
+        B[4] = dt * (-arm / Jx);
+        B[5] = dt * (-arm / Jy);
+        B[6] = dt * (arm / Jy);
+        B[7] = dt * (km / Jz);
+        B[8] = dt * (-km / Jz);
+        // c = s + dt f - A s - B u over the entries that are not 0, in column order
+        T c[NS];
+#pragma unroll
+        for (int i = 0; i < NS; ++i) c[i] = st[i] + dt * f[i];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            c[i] -= st[i];
+            c[i] -= dt * st[3 + i];
+            c[3 + i] -= st[3 + i];
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                if (i < 2 || k < 2) c[3 + i] -= A[i * 3 + k] * st[6 + k];
+#pragma unroll
+            for (int k = 0; k < NU; ++k) c[3 + i] -= B[i] * ut[k];
+        }
+        c[6] -= A[8] * st[6];
+        c[6] -= A[9] * st[7];
+        c[6] -= dt * st[9];
+        c[6] -= A[10] * st[10];
+        c[6] -= A[11] * st[11];
+        c[7] -= A[12] * st[6];
+        c[7] -= st[7];
+        c[7] -= A[13] * st[10];
+        c[7] -= A[14] * st[11];
+        c[8] -= A[15] * st[6];
+        c[8] -= A[16] * st[7];
+        c[8] -= st[8];
+        c[8] -= A[17] * st[10];
+        c[8] -= A[18] * st[11];
+        c[9] -= st[9];
+        c[9] -= A[19] * st[10];
+        c[9] -= A[20] * st[11];
+        c[9] -= B[3] * ut[1];
+        c[9] -= B[4] * ut[3];
+        c[10] -= A[21] * st[9];
+        c[10] -= st[10];
+        c[10] -= A[22] * st[11];
+        c[10] -= B[5] * ut[0];
+        c[10] -= B[6] * ut[2];
+        c[11] -= A[23] * st[9];
+        c[11] -= A[24] * st[10];
+        c[11] -= st[11];
+        c[11] -= B[7] * ut[0];
+        c[11] -= B[8] * ut[1];
+        c[11] -= B[7] * ut[2];
+        c[11] -= B[8] * ut[3];
+#pragma unroll
+        for (int i = 0; i < 25; ++i) rec[Mp::rA + i] = F(A[i]);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) rec[Mp::rB + i] = F(B[i]);
+#pragma unroll
+        for (int i = 0; i < NS; ++i) rec[Mp::rc + i] = F(c[i]);
+#pragma unroll
+        for (int i = 0; i < NU; ++i) {
+            T acc = -a.damp * ut[i];
+            if (bounded(m.u_lo[i], m.u_hi[i])) acc -= a.rho_box * (src.zu[ku + i] - src.wu[ku + i]);
+            rec[Mp::rr + i] = F(acc);
+        }
+    }
+    // diagonal and linear terms, and the 6 x 6 Gauss-Newton block over (position, angles)
+    T Qd[NS], qr[NS], H[6][6];
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        Qd[i] = T(2) * m.Qs[i];
+        qr[i] = -T(2) * m.Qs[i] * a.s_ref[ks + i];
+        if (t >= 1) {
+            Qd[i] += a.damp;
+            qr[i] -= a.damp * st[i];
+            if (bounded(m.s_lo[i], m.s_hi[i])) {
+                Qd[i] += a.rho_box;
+                qr[i] -= a.rho_box * (src.zs[ks + i] - src.ws[ks + i]);
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 6; ++i)
+#pragma unroll
+        for (int k = 0; k < 6; ++k) H[i][k] = T(0);
+    if (t >= 1) {
+        for (int part = 0; part < sm.NP; ++part) {
+            const int gp = sm.part0 + part;
+            const long long col = sm.qbeg + part * N + (t - 1);
+            T W[3][3], Wc[3], E[9], off[3], rho[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) off[i] = a.g.part_off[gp * 3 + i];
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int k = 0; k <= i; ++k) W[i][k] = W[k][i] = src.stats[(long long)(i * (i + 1) / 2 + k) * a.Qtot + col];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) Wc[i] = src.stats[(long long)(6 + i) * a.Qtot + col];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) E[i] = src.stats[(long long)(9 + i) * a.Qtot + col];
+            T gv[3], WR[9];  // Wc - W rho, W R
+#pragma unroll
+            for (int i = 0; i < 3; ++i) rho[i] = st[i] + R[i * 3] * off[0] + R[i * 3 + 1] * off[1] + R[i * 3 + 2] * off[2];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                gv[i] = Wc[i] - W[i][0] * rho[0] - W[i][1] * rho[1] - W[i][2] * rho[2];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) WR[i * 3 + k] = W[i][0] * R[k] + W[i][1] * R[3 + k] + W[i][2] * R[6 + k];
+            }
+            T Hp[6][6], g[6];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                g[i] = -gv[i];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) Hp[i][k] = W[i][k];
+            }
+#pragma unroll
+            for (int x = 0; x < 3; ++x) {
+                T d[3], Wd[3], WD[9];  // drho/dangle_x, W d, W dR_x
+#pragma unroll
+                for (int i = 0; i < 3; ++i) d[i] = dR[x][i * 3] * off[0] + dR[x][i * 3 + 1] * off[1] + dR[x][i * 3 + 2] * off[2];
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    Wd[i] = W[i][0] * d[0] + W[i][1] * d[1] + W[i][2] * d[2];
+                    Hp[i][3 + x] = Wd[i];
+#pragma unroll
+                    for (int k = 0; k < 3; ++k)
+                        WD[i * 3 + k] = W[i][0] * dR[x][k] + W[i][1] * dR[x][3 + k] + W[i][2] * dR[x][6 + k];
+                }
+                T gx = -(d[0] * gv[0] + d[1] * gv[1] + d[2] * gv[2]);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) gx += dR[x][i] * (E[i] + WR[i]);
+                g[3 + x] = gx;
+#pragma unroll
+                for (int y = 0; y <= x; ++y) {
+                    T v = T(0);
+#pragma unroll
+                    for (int i = 0; i < 3; ++i)
+                        v += (dR[y][i * 3] * off[0] + dR[y][i * 3 + 1] * off[1] + dR[y][i * 3 + 2] * off[2]) * Wd[i];
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) v += dR[y][i] * WD[i];
+                    Hp[3 + y][3 + x] = v;
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 6; ++i) {
+                T hs = T(0);
+#pragma unroll
+                for (int k = 0; k < 6; ++k) {
+                    const T h = i <= k ? Hp[i][k] : Hp[k][i];
+                    hs += h * st[k < 3 ? k : 3 + k];
+                    if (i <= k) H[i][k] += a.sigma * h;
+                }
+                qr[i < 3 ? i : 3 + i] += a.sigma * (g[i] - hs);
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        rec[Mp::rq + i] = F(qr[i]);
+#pragma unroll
+        for (int k = i; k < NS; ++k) {
+            const bool ci = i < 3 || (i >= 6 && i < 9), ck = k < 3 || (k >= 6 && k < 9);
+            T v = i == k ? Qd[i] : T(0);
+            if (ci && ck) v += H[i < 3 ? i : i - 3][k < 3 ? k : k - 3];
+            rec[Mp::rQ + Mp::sym(i, k)] = F(v);
+        }
+    }
+}
 
 template <typename T, typename F, int KIND>
 __global__ void __launch_bounds__(kTrajBlock) k_traj_stage(RicArgs<T> a) {
@@ -407,38 +514,42 @@ __global__ void __launch_bounds__(kTrajBlock) k_traj_stage(RicArgs<T> a) {
     StageParams<T> sp;
     StageSrc<T> src;
     stage_inputs(a, sp, src);
-    struct Sink {
-        F *r;
-        __device__ void A(int i, int k, T v) {
-            const int e = RicSparse<KIND>::a_slot(i, k);
-            if (e >= 0) r[Mp::rA + e] = F(v);
+    if constexpr (KIND == 2) {
+        for (int t = lane; t <= sm.N; t += NT) quad_record<T, F>(sp, src, sm, t, scr + Mp::rec(t));
+    } else {
+        struct Sink {
+            F *r;
+            __device__ void A(int i, int k, T v) {
+                const int e = RicSparse<KIND>::a_slot(i, k);
+                if (e >= 0) r[Mp::rA + e] = F(v);
+            }
+            __device__ void B(int i, int k, T v) {
+                const int e = RicSparse<KIND>::b_slot(i, k);
+                if (e >= 0) r[Mp::rB + e] = F(v);
+            }
+            __device__ void c(int i, T v) { r[Mp::rc + i] = F(v); }
+            __device__ void u(int i, T v) { r[Mp::rr + i] = F(v); }
+            __device__ void Q(int i, int k, T v) {
+                if (i <= k) r[Mp::rQ + Mp::sym(i, k)] = F(v);
+            }
+            __device__ void q(int i, T v) { r[Mp::rq + i] = F(v); }
+        };
+        // records through shared memory (odd stride): written straight to the scratch,
+        // every 8-byte store of a warp touches 32 sectors
+        constexpr int RS = traj_rec_stride<F, KIND>();
+        extern __shared__ __align__(16) unsigned char smem_raw[];
+        F *rec = reinterpret_cast<F *>(smem_raw);  // [NT][RS]
+        for (int t0 = 0; t0 <= sm.N; t0 += NT) {
+            const int n = min(NT, sm.N + 1 - t0);
+            if (lane < n) {
+                Sink out{rec + lane * RS};
+                assemble_terms<T, KIND>(sp, src, sm, t0 + lane, out);
+            }
+            __syncthreads();
+            F *dst = scr + Mp::rec(t0);
+            for (int e = lane; e < n * Mp::REC; e += NT) dst[e] = rec[e / Mp::REC * RS + e % Mp::REC];
+            __syncthreads();
         }
-        __device__ void B(int i, int k, T v) {
-            const int e = RicSparse<KIND>::b_slot(i, k);
-            if (e >= 0) r[Mp::rB + e] = F(v);
-        }
-        __device__ void c(int i, T v) { r[Mp::rc + i] = F(v); }
-        __device__ void u(int i, T v) { r[Mp::rr + i] = F(v); }
-        __device__ void Q(int i, int k, T v) {
-            if (i <= k) r[Mp::rQ + Mp::sym(i, k)] = F(v);
-        }
-        __device__ void q(int i, T v) { r[Mp::rq + i] = F(v); }
-    };
-    // records through shared memory (odd stride): written straight to the scratch,
-    // every 8-byte store of a warp touches 32 sectors
-    constexpr int RS = traj_rec_stride<F, KIND>();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    F *rec = reinterpret_cast<F *>(smem_raw);  // [NT][RS]
-    for (int t0 = 0; t0 <= sm.N; t0 += NT) {
-        const int n = min(NT, sm.N + 1 - t0);
-        if (lane < n) {
-            Sink out{rec + lane * RS};
-            assemble_terms<T, KIND>(sp, src, sm, t0 + lane, out);
-        }
-        __syncthreads();
-        F *dst = scr + Mp::rec(t0);
-        for (int e = lane; e < n * Mp::REC; e += NT) dst[e] = rec[e / Mp::REC * RS + e % Mp::REC];
-        __syncthreads();
     }
     if (lane < NS) scr[Mp::s0(sm.N) + lane] = F(a.s[(long long)sm.state0 * NS + lane]);
 }
@@ -609,6 +720,135 @@ __global__ void __launch_bounds__(32 * kLqWarps) k_traj_lq(LqArgs2<F> a) {
     }
 }
 
+// The 12-state model: one CTA of four warps (one per scheduler) per scenario.  Per
+// stage 7 + 7 + 6 FP64 instructions of the three products on every warp and 29 of the
+// 4 x 4 system on the first (Gauss-Jordan, a column of [Quu | Qus qu] per lane; dense
+// products took 24 + 24 + 4 and the inverse about 60).  The sweep splits each of the
+// 16 rows of [F; K] over two lanes.  One step of 64 scenarios of horizon 40 takes 31 +
+// 134 + 10 us in the three kernels (390 in one kernel of dense products), 256 of
+// horizon 16 take 30 + 62 + 10 (239).
+template <typename F>
+__global__ void __launch_bounds__(128) k_traj_lq4(LqArgs2<F> a) {
+    using Mp = RicMap<2>;
+    constexpr int NS = Mp::NS, NU = Mp::NU, NZ = Mp::NZ, REC = Mp::REC, OUT = Mp::OUT, NT = 128;
+    constexpr int PR = (REC + NT - 1) / NT, PO = (OUT + NT - 1) / NT;
+    __shared__ F sm[Mp::SIZE];
+    const int tid = threadIdx.x, lane = tid & 31, s = a.order[blockIdx.x];
+    if (blockIdx.x == 0 && tid == 0) *a.iter += 1;
+    if (a.scen_status[s] != kActive) return;
+    const int N = a.meta[s].N;
+    F *scr = reinterpret_cast<F *>(a.scratch) + a.scratch0[s];
+    typename LqSlotsOf<F, std::remove_cv_t<decltype(kRicTab<2, NT, 0>)>>::type prod_y;
+    typename LqSlotsOf<F, std::remove_cv_t<decltype(kRicTab<2, NT, 1>)>>::type prod_m;
+    typename LqSlotsOf<F, std::remove_cv_t<decltype(kRicTab<2, NT, 2>)>>::type prod_p;
+    prod_y.load(kRicTab<2, NT, 0>, tid, sm);
+    prod_m.load(kRicTab<2, NT, 1>, tid, sm);
+    prod_p.load(kRicTab<2, NT, 2>, tid, sm);
+    int om[PO];
+#pragma unroll
+    for (int r = 0; r < PO; ++r) om[r] = tid + NT * r < OUT ? kRicOut<2>.at[tid + NT * r] : 0;
+    if (tid == 0) {
+        sm[Mp::ZERO] = F(0);
+        sm[Mp::ONE] = F(1);
+        sm[Mp::DT] = a.dt;
+        for (int x = 0; x < NU; ++x) sm[Mp::RU + x] = a.ru[x];
+    }
+    const F *rN = scr + Mp::rec(N), *r1 = scr + Mp::rec(N - 1);
+    for (int e = tid; e < Mp::NSYM; e += NT) sm[Mp::P0 + e] = rN[Mp::rQ + e];
+    for (int e = tid; e < NS; e += NT) sm[Mp::p0 + e] = rN[Mp::rq + e];
+    for (int e = tid; e < REC; e += NT) sm[Mp::REC0 + e] = r1[e];
+    bool ok = true;
+    for (int t = N - 1; t >= 0; --t) {
+        F nxt[PR];
+        __syncthreads();
+        if (t >= 1) {
+            const F *rn = scr + Mp::rec(t - 1);
+#pragma unroll
+            for (int r = 0; r < PR; ++r)
+                if (tid + NT * r < REC) nxt[r] = rn[tid + NT * r];
+        }
+        prod_y.run();
+        __syncthreads();
+        prod_m.run();
+        __syncthreads();
+        if (tid < 32) {
+            // [K | k] = -Quu^-1 [Qus | qu]: lane c < 4 holds column c of Quu, lane 4 + j
+            // column j of [Qus | qu].  Quu is positive definite iff every pivot is
+            // positive; 1 takes the place of one that is not, the scenario fails.
+            const int j = lane - NU;
+            F v[NU];
+#pragma unroll
+            for (int i = 0; i < NU; ++i)
+                v[i] = sm[lane < NU ? Mp::U0 + (i <= lane ? i * NU + lane : lane * NU + i) : Mp::H0 + i * (NS + 1) + min(j, NS)];
+            if (j == NS)
+#pragma unroll
+                for (int i = 0; i < NU; ++i) v[i] += sm[Mp::HQ1 + i];
+#pragma unroll
+            for (int c = 0; c < NU; ++c) {
+                F col[NU];
+#pragma unroll
+                for (int i = 0; i < NU; ++i) col[i] = __shfl_sync(0xffffffffu, v[i], c);
+                const bool pd = lq_positive(col[c]);
+                ok = ok && pd;
+                v[c] *= pd ? lq_rcp(col[c]) : F(1);
+#pragma unroll
+                for (int i = 0; i < NU; ++i)
+                    if (i != c) v[i] = fma(-col[i], v[c], v[i]);
+            }
+            if (j >= 0 && j <= NS)
+#pragma unroll
+                for (int i = 0; i < NU; ++i) sm[Mp::K0 + i * (NS + 1) + j] = -v[i];
+        }
+        __syncthreads();
+        prod_p.run();
+        __syncthreads();
+        F *o = scr + Mp::out(N, t);
+#pragma unroll
+        for (int r = 0; r < PO; ++r)
+            if (tid + NT * r < OUT) o[tid + NT * r] = sm[om[r]];
+        __syncthreads();
+        if (t >= 1) {
+#pragma unroll
+            for (int r = 0; r < PR; ++r)
+                if (tid + NT * r < REC) sm[Mp::REC0 + tid + NT * r] = nxt[r];
+        }
+    }
+    __syncthreads();  // the outputs of every thread are visible to the sweep
+    if (tid >= 32) return;
+    // forward sweep: lanes i and 16 + i own row i of [F; K], half of the sum each
+    constexpr int AHEAD = 4, HN = NS / 2;
+    const int i = lane & 15, half = lane >> 4;
+    F x = i < NS ? scr[Mp::s0(N) + i] : F(0);
+    F row[AHEAD][HN], fv[AHEAD];
+    auto fetch = [&](int t, F (&r)[HN], F &f) {
+        const F *o = scr + Mp::out(N, min(t, N - 1));
+#pragma unroll
+        for (int k = 0; k < HN; ++k) r[k] = o[i * NS + half * HN + k];
+        f = half ? F(0) : o[NZ * NS + i];
+    };
+#pragma unroll
+    for (int d = 0; d < AHEAD; ++d) fetch(d, row[d], fv[d]);
+    bool fin = true;
+    for (int t0 = 0; t0 < N; t0 += AHEAD) {
+#pragma unroll
+        for (int d = 0; d < AHEAD; ++d) {
+            const int t = t0 + d;
+            F v = fv[d];
+#pragma unroll
+            for (int k = 0; k < HN; ++k) v = fma(row[d][k], __shfl_sync(0xffffffffu, x, half * HN + k), v);
+            v += __shfl_xor_sync(0xffffffffu, v, 16);
+            x = v;
+            if (t < N) {
+                if (!half) scr[Mp::sol(N, t) + i] = v;
+                fin = fin && lq_finite(v);
+            }
+            fetch(t + AHEAD, row[d], fv[d]);
+        }
+    }
+    const bool good = __all_sync(0xffffffffu, ok && fin);
+    if (lane == 0) a.ok[s] = good;
+}
+
 // s, u from the sweep, then the box block and the poses of the new iterate
 template <typename T, typename F, int KIND>
 __global__ void __launch_bounds__(kTrajBlock) k_traj_apply(RicArgs<T> a, const int *lq_ok) {
@@ -672,16 +912,20 @@ cudaError_t launch_traj(const RicArgs<T> &a, int *lq_ok, const int *order, int m
     l.scratch = a.scratch;
     l.scratch0 = a.scratch0;
     l.dt = F(a.model.dt);
-    for (int i = 0; i < 2; ++i)
+    for (int i = 0; i < MDims<KIND>::NU; ++i)
         l.ru[i] = F(2) * F(a.model.Qu[i]) + F(a.damp) +
                   (a.model.u_lo[i] > T(-1e29) || a.model.u_hi[i] < T(1e29) ? F(a.rho_box) : F(0));
     l.ok = lq_ok;
     l.iter = a.iter;
     const int steps = std::min(kTrajBlock, (max_n + 1 + 31) / 32 * 32);
     k_traj_stage<T, F, KIND><<<a.n_scen, steps, sizeof(F) * steps * traj_rec_stride<F, KIND>(), st>>>(a);
-    const int one = a.n_scen <= 4 * n_sm, groups = one ? a.n_scen : (a.n_scen + 1) / 2, ctas = std::min(n_sm, groups);
-    if (one) k_traj_lq<F, KIND, 32><<<ctas, 32 * kLqWarps, 0, st>>>(l);
-    else k_traj_lq<F, KIND, 16><<<ctas, 32 * kLqWarps, 0, st>>>(l);
+    if constexpr (KIND == 2) {
+        k_traj_lq4<F><<<a.n_scen, 128, 0, st>>>(l);
+    } else {
+        const int one = a.n_scen <= 4 * n_sm, groups = one ? a.n_scen : (a.n_scen + 1) / 2, ctas = std::min(n_sm, groups);
+        if (one) k_traj_lq<F, KIND, 32><<<ctas, 32 * kLqWarps, 0, st>>>(l);
+        else k_traj_lq<F, KIND, 16><<<ctas, 32 * kLqWarps, 0, st>>>(l);
+    }
     k_traj_apply<T, F, KIND><<<a.n_scen, steps, 0, st>>>(a, lq_ok);
     return cudaGetLastError();
 }
@@ -691,11 +935,7 @@ cudaError_t launch_riccati_f(const RicArgs<T> &a, int *lq_ok, const int *order, 
     switch (a.model.kind) {
         case 0: return launch_traj<T, F, 0>(a, lq_ok, order, max_n, n_sm, st);
         case 1: return launch_traj<T, F, 1>(a, lq_ok, order, max_n, n_sm, st);
-        case 2: {
-            k_riccati<T, F, 2, 128><<<a.n_scen, 128, 0, st>>>(a);
-            k_advance<<<1, 1, 0, st>>>(a.iter);
-            return cudaGetLastError();
-        }
+        case 2: return launch_traj<T, F, 2>(a, lq_ok, order, max_n, n_sm, st);
     }
     return cudaErrorInvalidValue;
 }

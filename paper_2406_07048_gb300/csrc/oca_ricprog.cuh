@@ -47,6 +47,20 @@ template <> struct RicSparse<1> {
     }
     OCA_HD static constexpr int b_slot(int i, int k) { return k == 1 ? (i == 2 ? 0 : i == 4 ? 1 : -1) : -1; }
 };
+// 12-state quadrotor: positions and velocities, ZYX angles (6..8), body rates.  The
+// thrust column of B is the same for the four rotors.
+template <> struct RicSparse<2> {
+    static constexpr int NA = 29, NB = 20, REC_A = 25, REC_B = 9;
+    static constexpr SpEntry A[NA] = {{0, 3, -1}, {1, 4, -1}, {2, 5, -1},
+                                      {3, 6, 0}, {3, 7, 1}, {3, 8, 2}, {4, 6, 3}, {4, 7, 4}, {4, 8, 5}, {5, 6, 6}, {5, 7, 7},
+                                      {6, 6, 8}, {6, 7, 9}, {6, 9, -1}, {6, 10, 10}, {6, 11, 11},
+                                      {7, 6, 12}, {7, 10, 13}, {7, 11, 14},
+                                      {8, 6, 15}, {8, 7, 16}, {8, 10, 17}, {8, 11, 18},
+                                      {9, 10, 19}, {9, 11, 20}, {10, 9, 21}, {10, 11, 22}, {11, 9, 23}, {11, 10, 24}};
+    static constexpr SpEntry B[NB] = {{3, 0, 0}, {3, 1, 0}, {3, 2, 0}, {3, 3, 0}, {4, 0, 1}, {4, 1, 1}, {4, 2, 1}, {4, 3, 1},
+                                      {5, 0, 2}, {5, 1, 2}, {5, 2, 2}, {5, 3, 2}, {9, 1, 3}, {9, 3, 4}, {10, 0, 5}, {10, 2, 6},
+                                      {11, 0, 7}, {11, 1, 8}, {11, 2, 7}, {11, 3, 8}};
+};
 template <int KIND>
 constexpr bool ric_slots_agree() {
     using SP = RicSparse<KIND>;
@@ -75,6 +89,8 @@ struct RicMap {
     static constexpr int NS = MDims<KIND>::NS, NU = MDims<KIND>::NU;
     using SP = RicSparse<KIND>;
     static constexpr int NSYM = NS * (NS + 1) / 2;
+    // long products with vectors (P c + p, A^T w, B^T w) are summed in WS parts
+    static constexpr int WS = NS > 6 ? 2 : 1;
     static constexpr int rA = 0, rB = SP::REC_A, rc = rB + SP::REC_B, rq = rc + NS, rr = rq + NS, rQ = rr + NU;
     static constexpr int REC = (rQ + NSYM + 1) & ~1;
     // shared region
@@ -82,11 +98,12 @@ struct RicMap {
     static constexpr int P0 = REC0 + REC, p0 = P0 + NSYM;
     static constexpr int Y0 = p0 + NS;           // Y[k][j] = (P A)[k][j], row-major (columns equal to P's are not formed)
     static constexpr int YB0 = Y0 + NS * NS;     // (P B)[k][x], only the rows that B touches
-    static constexpr int W0 = YB0 + NS * NU;     // P c + p
-    static constexpr int M0 = W0 + NS;           // Qss, upper triangle
-    static constexpr int H0 = M0 + NSYM;         // Qus [x][j], then qu [x] in column NS
-    static constexpr int G0 = H0 + NU * (NS + 1);  // qs
-    static constexpr int U0 = G0 + NS;           // Quu, row-major upper
+    static constexpr int W0 = YB0 + NS * NU;     // P c + p [part][k]
+    static constexpr int M0 = W0 + WS * NS;      // Qss, upper triangle
+    static constexpr int H0 = M0 + NSYM;         // Qus [x][j], then qu [x] (its first part) in column NS
+    static constexpr int HQ1 = H0 + NU * (NS + 1);  // qu's second part [x]
+    static constexpr int G0 = HQ1 + (WS - 1) * NU;  // qs [part][i]
+    static constexpr int U0 = G0 + WS * NS;      // Quu, row-major upper
     static constexpr int K0 = U0 + NU * NU;      // K [x][j], k [x] in column NS
     static constexpr int F0 = K0 + NU * (NS + 1);  // F = A + B K (rows that B touches), then f in column NS
     static constexpr int SIZE = F0 + NS * (NS + 1);
@@ -181,9 +198,11 @@ struct RicBuild {
                     if (SP::B[i].col == x) term(o, b_src(i), Mp::P0 + Mp::sym(k, SP::B[i].row));
                 add(l, o);
             }
-            RicOp o = start(Mp::p0 + k, Mp::W0 + k);
-            for (int i = 0; i < NS; ++i) term(o, Mp::REC0 + Mp::rc + i, Mp::P0 + Mp::sym(k, i));
-            add(l, o);
+            for (int w = 0; w < Mp::WS; ++w) {
+                RicOp o = start(w == 0 ? Mp::p0 + k : Mp::ZERO, Mp::W0 + w * NS + k);
+                for (int i = w * NS / Mp::WS; i < (w + 1) * NS / Mp::WS; ++i) term(o, Mp::REC0 + Mp::rc + i, Mp::P0 + Mp::sym(k, i));
+                add(l, o);
+            }
         }
         return l;
     }
@@ -204,15 +223,23 @@ struct RicBuild {
                 at_terms(o, i, 0, 0, j);
                 add(l, o);
             }
-            RicOp o = start(Mp::REC0 + Mp::rq + i, Mp::G0 + i);
-            at_terms(o, i, Mp::W0, 1, -1);
-            add(l, o);
+            for (int w = 0; w < Mp::WS; ++w) {
+                RicOp o = start(w == 0 ? Mp::REC0 + Mp::rq + i : Mp::ZERO, Mp::G0 + w * NS + i);
+                at_terms(o, i, Mp::W0 + w * NS, 1, -1);
+                add(l, o);
+            }
         }
         for (int x = 0; x < NU; ++x) {
             for (int j = 0; j <= NS; ++j) {
                 RicOp o = start(j < NS ? Mp::ZERO : Mp::REC0 + Mp::rr + x, Mp::H0 + x * (NS + 1) + j);
                 for (int i = 0; i < SP::NB; ++i)
                     if (SP::B[i].col == x) term(o, b_src(i), j < NS ? Yat(SP::B[i].row, j) : Mp::W0 + SP::B[i].row);
+                add(l, o);
+            }
+            if (Mp::WS > 1) {
+                RicOp o = start(Mp::ZERO, Mp::HQ1 + x);
+                for (int i = 0; i < SP::NB; ++i)
+                    if (SP::B[i].col == x) term(o, b_src(i), Mp::W0 + NS + SP::B[i].row);
                 add(l, o);
             }
             for (int y = x; y < NU; ++y) {
@@ -234,6 +261,7 @@ struct RicBuild {
                 add(l, o);
             }
             RicOp o = start(Mp::G0 + i, Mp::p0 + i);
+            if (Mp::WS > 1) term(o, Mp::ONE, Mp::G0 + NS + i);
             for (int x = 0; x < NU; ++x) term(o, Mp::H0 + x * (NS + 1) + i, Mp::K0 + x * (NS + 1) + NS);
             add(l, o);
         }

@@ -100,7 +100,7 @@ static void test() {
         }
         double v = q[i];
         for (int l = 0; l < NS; ++l) v += A[l][i] * w[l];
-        check(sm[Mp::G0 + i], v, "qs");
+        check(sm[Mp::G0 + i] + (Mp::WS > 1 ? sm[Mp::G0 + NS + i] : 0.0), v, "qs");
     }
     for (int x = 0; x < NU; ++x) {
         for (int j = 0; j < NS; ++j) {
@@ -110,7 +110,7 @@ static void test() {
         }
         double v = r[x];
         for (int l = 0; l < NS; ++l) v += B[l][x] * w[l];
-        check(sm[Mp::H0 + x * (NS + 1) + NS], v, "qu");
+        check(sm[Mp::H0 + x * (NS + 1) + NS] + (Mp::WS > 1 ? sm[Mp::HQ1 + x] : 0.0), v, "qu");
         for (int y = x; y < NU; ++y) {
             double u = x == y ? 5.0 + x : 0.0;
             for (int l = 0; l < NS; ++l)
@@ -130,7 +130,7 @@ static void test() {
             for (int x = 0; x < NU; ++x) v += H(x, i) * K(x, j);
             check(sm[Mp::P0 + Mp::sym(i, j)], v, "P");
         }
-        double v = old[Mp::G0 + i];
+        double v = old[Mp::G0 + i] + (Mp::WS > 1 ? old[Mp::G0 + NS + i] : 0.0);
         for (int x = 0; x < NU; ++x) v += H(x, i) * K(x, NS);
         check(sm[Mp::p0 + i], v, "p");
     }
@@ -154,5 +154,6 @@ int main() {
     test<0, 32>();
     test<1, 16>();
     test<1, 32>();
+    test<2, 128>();
     return 0;
 }

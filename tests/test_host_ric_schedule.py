@@ -23,4 +23,4 @@ def test_recursion_schedules_match_dense_products_on_host(tmp_path):
     print(out.stdout)
     assert out.returncode == 0, out.stdout
     seen = {tuple(int(v) for v in line.split()[:2]) for line in out.stdout.split("\n") if line.strip()}
-    assert seen == {(0, 16), (0, 32), (1, 16), (1, 32)}
+    assert seen == {(0, 16), (0, 32), (1, 16), (1, 32), (2, 128)}
