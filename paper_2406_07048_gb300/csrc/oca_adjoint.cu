@@ -770,7 +770,7 @@ __global__ void __launch_bounds__(256) k_adj_alpha(AdjAlphaArgs<T> a) {
         const long long p = sm.pair0 + (long long)j * Q + qc;
         int bas[D + 1];
         T xB[D + 1], alpha, x[D];
-        lp_solve<T, D>(L, bas, xB, alpha);
+        lp_solve<T, D>(LaneCols<T, D>(L), bas, xB, alpha);
         const bool okx = lp_primal<T, D>(L, bas, x);
         const T ga = valid && okx ? a.grad_alpha[p] : T(0);
         T w[D];

@@ -125,8 +125,11 @@ __global__ void k_mpc_plant(MpcArgs<T> a, int n_scen) {
 
 // collision of the true state with every obstacle: alpha* < 1 for some
 // (part, obstacle) marks the scenario with the first step it happened
+// One thread per (obstacle, part) with its LP columns staged in shared memory (at most
+// 32 KB), 32 threads a block: a latency chain of a few pivots, so the blocks spread.
+constexpr int kCollideThreads = 32;
 template <typename T, int KIND>
-__global__ void k_mpc_collide(MpcArgs<T> a) {
+__global__ void __launch_bounds__(kCollideThreads) k_mpc_collide(MpcArgs<T> a) {
     constexpr int NS = MDims<KIND>::NS, D = MDims<KIND>::D;
     const int s = blockIdx.y;
     const ScenMeta sm = a.meta[s];
@@ -149,7 +152,12 @@ __global__ void k_mpc_collide(MpcArgs<T> a) {
     L.no = a.g.obs_nf[gm];
     int bas[D + 1];
     T xB[D + 1], alpha;
-    lp_solve<T, D>(L, bas, xB, alpha);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T *rec = reinterpret_cast<T *>(smem_raw) + threadIdx.x * kLpRec;
+    const int stride = kCollideThreads * kLpRec;
+    lp_stage_part<T, D>(L, rec, stride);
+    lp_stage_obstacle<T, D>(L, rec, stride);
+    lp_solve<T, D>(StagedCols<T, D>{rec, stride, L.nr, L.no}, bas, xB, alpha);
     if (alpha < T(1)) atomicCAS(a.collided + s, -1, a.c + 1);
 }
 
@@ -159,7 +167,10 @@ cudaError_t mpc_launch_t(const MpcArgs<T> &a, int stage, int n_scen, int max_blk
         case 0: k_mpc_window<T, KIND><<<n_scen, 32, 0, st>>>(a); break;
         case 1: k_mpc_shift_pairs<T><<<dim3((max_blk + kShiftWarps - 1) / kShiftWarps, n_scen), 32 * kShiftWarps, 0, st>>>(a, MDims<KIND>::D); break;
         case 2: k_mpc_plant<T, KIND><<<(n_scen + 63) / 64, 64, 0, st>>>(a, n_scen); break;
-        default: k_mpc_collide<T, KIND><<<dim3((max_blk + 63) / 64, n_scen), 64, 0, st>>>(a); break;
+        default:
+            k_mpc_collide<T, KIND><<<dim3((max_blk + kCollideThreads - 1) / kCollideThreads, n_scen), kCollideThreads,
+                                     sizeof(T) * kLpRec * kCollideThreads * (a.g.FR + a.g.FO), st>>>(a);
+            break;
     }
     return cudaGetLastError();
 }

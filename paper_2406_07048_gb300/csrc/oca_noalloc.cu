@@ -68,6 +68,9 @@ __global__ void k_scale_one(OneScen sc, Geom<T> g, const T *pose, T *alpha, T *l
     L.A = g.part_A + (long long)part * g.FR * D;
     L.b = g.part_b + (long long)part * g.FR;
     L.nr = g.part_nf[part];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T *rec = reinterpret_cast<T *>(smem_raw) + (size_t)warp * (g.FR + g.FO) * 32 * kLpRec + lane * kLpRec;
+    lp_stage_part<T, D>(L, rec, 32 * kLpRec);
     for (int j = warp; j < sc.M; j += W) {
         L.C = g.obs_C + (long long)j * g.FO * D;
         L.d = g.obs_d + (long long)j * g.FO;
@@ -75,7 +78,8 @@ __global__ void k_scale_one(OneScen sc, Geom<T> g, const T *pose, T *alpha, T *l
         const long long p = (long long)j * sc.Q + q;
         int bas[V];
         T xB[V], a;
-        int st = lp_solve<T, D>(L, bas, xB, a);
+        lp_stage_obstacle<T, D>(L, rec, 32 * kLpRec);
+        int st = lp_solve<T, D>(StagedCols<T, D>{rec, 32 * kLpRec, L.nr, L.no}, bas, xB, a);
         if (!(a == a)) st = OCA_PAIR_NONFINITE;
         alpha[p] = a;
         if (verdict) verdict[p] = a >= T(1) ? 1 : 0;
@@ -141,11 +145,17 @@ oca_status run(const oca_scene_desc *d, const oca_model *m, void *scratch, const
     if (cudaGetLastError() != cudaSuccess) return OCA_ERR_CUDA;
     const int W = sc.M >= 32 ? 4 : (sc.M >= 8 ? 2 : 1);
     const unsigned tiles = (unsigned)((sc.Q + 31) / 32);
+    const size_t sm = sizeof(T) * kLpRec * 32 * (size_t)W * (g.FR + g.FO);
+    if (sm > 48 * 1024 &&
+        cudaFuncSetAttribute(d->dim == 2 ? reinterpret_cast<const void *>(k_scale_one<T, 2>)
+                                         : reinterpret_cast<const void *>(k_scale_one<T, 3>),
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
+        return OCA_ERR_CUDA;
     if (d->dim == 2)
-        k_scale_one<T, 2><<<tiles, dim3(32, W), 0, st>>>(sc, g, pose, static_cast<T *>(alpha), static_cast<T *>(lambda),
+        k_scale_one<T, 2><<<tiles, dim3(32, W), sm, st>>>(sc, g, pose, static_cast<T *>(alpha), static_cast<T *>(lambda),
                                                         static_cast<T *>(mu), verdict, status);
     else
-        k_scale_one<T, 3><<<tiles, dim3(32, W), 0, st>>>(sc, g, pose, static_cast<T *>(alpha), static_cast<T *>(lambda),
+        k_scale_one<T, 3><<<tiles, dim3(32, W), sm, st>>>(sc, g, pose, static_cast<T *>(alpha), static_cast<T *>(lambda),
                                                         static_cast<T *>(mu), verdict, status);
     return cudaGetLastError() == cudaSuccess ? OCA_OK : OCA_ERR_CUDA;
 }

