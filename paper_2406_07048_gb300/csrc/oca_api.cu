@@ -1086,24 +1086,29 @@ oca_status oca_scene_create(oca_ctx *ctx, const oca_scene_desc *d, oca_scene **o
     for (int s = 0; s < S; ++s) by_horizon[s] = s;
     std::stable_sort(by_horizon.begin(), by_horizon.end(), [&](int x, int y) { return sc->meta[x].N > sc->meta[y].N; });
     // Warps per tile (until oca_scene_set_warps): as many as keep the launch within
-    // 2.5 times the warps that an SM holds (16, 12 in FP64 and 8 in 3-D of the pair
-    // kernel, 32 of the LP and margin kernels, by their registers), a power of two so
-    // that whole CTAs fill them, no more than obstacles.  Few tiles then spread their
-    // obstacles over idle SMs, many tiles amortise a warp's set-up over more of them.
+    // `waves` times the warps that an SM holds (16, 12 in FP64 or 3-D, 8 in both, of the
+    // pair kernel; 32 of the LP and margin kernels, by their registers), in counts whose
+    // CTAs fill them, no more than obstacles.  Few tiles then spread their obstacles over
+    // idle SMs, many tiles amortise a warp's set-up over more of them.
     // Pair kernel, us per launch: 5,660 trailer tiles 706 with 2 (773 with 5), 1,470
     // tiles 208 with 4 (251 with 2, 226 with 8), 345 tiles 74 with 16 (98 with 5), one
-    // tile of 4 obstacles in FP64 91 with 4 (264 with 1); LP kernel: 2,892 tiles 1,306
-    // with 4 (1,468 with 2), 4 tiles 100 with 16 (239 with 4); margin kernel: 5,660 tiles
-    // 1,107 with 4 (1,134 with 2).
-    auto pick = [&](int per_sm, int most, int least) {
-        int w = 16;
-        while (w > 1 && (w > most || (w > least && (double)tiles * w > 2.5 * per_sm * ctx->n_sm))) w /= 2;
-        return std::max(1, std::min(w, sc->maxM));
+    // tile of 4 obstacles in FP64 91 with 4 (264 with 1); in 3-D (equal tiles: one wave)
+    // 256 tiles 314 with 6 (389 with 8), 512 tiles 167 with 3 (177 with 8), 16 tiles 195
+    // with 8 (252 with 6).  LP kernel: 2,892 tiles 1,306 with 4 (1,468 with 2), 4 tiles
+    // 100 with 16 (239 with 4); margin kernel: 5,660 tiles 1,107 with 4 (1,134 with 2).
+    auto pick = [&](int per_sm, int most, int least, double waves) {
+        const int counts[] = {16, 8, 6, 4, 3, 2, 1};
+        for (int w : counts) {
+            if (w > most || (w % 3 == 0 && per_sm % 3 != 0)) continue;
+            if (w <= least || (double)tiles * w <= waves * per_sm * ctx->n_sm) return std::max(1, std::min(w, sc->maxM));
+        }
+        return 1;
     };
-    const int pair_warps = pair_max_warps(d->dim, dsize(d->dtype));
-    sc->W = pick(pair_warps, pair_warps, 2);
+    const size_t es = dsize(d->dtype);
+    const bool one_wave = d->dim == 3 && es == 4;
+    sc->W = pick(pair_sm_warps(d->dim, es), pair_max_warps(d->dim, es), one_wave ? 1 : 2, one_wave ? 1.0 : 2.5);
     while (sc->W > 1 && !warps_fit(sc, sc->W)) --sc->W;
-    sc->W_lp = pick(32, 16, 4);
+    sc->W_lp = pick(32, 16, 4, 2.5);
 
     const size_t ts = dsize(d->dtype);
     const int PK = d->dim + d->dim * d->dim;

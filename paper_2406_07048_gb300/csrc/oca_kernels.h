@@ -11,8 +11,10 @@ cudaError_t launch_pose(const PoseArgs<T> &a, int maxQ, cudaStream_t st);
 template <typename T>
 cudaError_t launch_pair(const PairArgs<T> &a, int dim, int mode, int solver, int n_tiles, int W, cudaStream_t st);
 
-// largest warps per tile the pair kernels are compiled for (their launch bound)
+// largest warps per tile the pair kernels accept
 int pair_max_warps(int dim, size_t es);
+// warps of the pair kernel that an SM holds (by its registers)
+int pair_sm_warps(int dim, size_t es);
 // dynamic shared memory of a pair-kernel launch with W warps per tile
 size_t pair_smem_bytes(int dim, size_t es, int W, int mode, int solver, int FR, int FO);
 

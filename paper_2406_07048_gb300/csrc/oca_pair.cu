@@ -60,11 +60,13 @@ __global__ void k_pose(PoseArgs<T> a) {
 #ifndef OCA_PAIR_MIN_BLOCKS
 #define OCA_PAIR_MIN_BLOCKS 1
 #endif
-// Launch bound of the pair kernel: 512 threads (16 warps) at most per CTA
-// for the FP32 2-D kernel, whose state fits 128 registers per thread without
-// spilling (16 resident warps per SM); 384 for the FP64 2-D kernel (about 165
-// registers); the 3-D kernel (4 x 4 Newton systems, up to 8 robot faces)
-// needs about 245 and is bounded at 256 threads.
+// Launch bound of the pair kernel, which sets its registers and with them the resident
+// warps per SM: 512 threads for the FP32 2-D kernel, whose state fits 128 registers
+// without spilling (16 warps); 384 for the FP64 2-D kernel (about 165 registers, 12
+// warps) and for the FP32 3-D kernel (4 x 4 Newton systems, up to 8 robot faces: 168
+// registers with a few spilled, 12 warps -- 64 quadrotor scenes 376 -> 314 us per launch
+// against 245 registers and 8 warps; 128 registers spill too much: 374 us); 256 for the
+// FP64 3-D kernel.
 #ifndef OCA_PAIR_MAX_THREADS_2D
 #define OCA_PAIR_MAX_THREADS_2D 512
 #endif
@@ -72,12 +74,16 @@ __global__ void k_pose(PoseArgs<T> a) {
 #define OCA_PAIR_MAX_THREADS_2D_F64 384
 #endif
 #ifndef OCA_PAIR_MAX_THREADS_3D
-#define OCA_PAIR_MAX_THREADS_3D 256
+#define OCA_PAIR_MAX_THREADS_3D 384
+#endif
+#ifndef OCA_PAIR_MAX_THREADS_3D_F64
+#define OCA_PAIR_MAX_THREADS_3D_F64 256
 #endif
 template <typename T, int D>
 struct PairBound {
     static constexpr int threads =
-        D == 3 ? OCA_PAIR_MAX_THREADS_3D : (sizeof(T) == 4 ? OCA_PAIR_MAX_THREADS_2D : OCA_PAIR_MAX_THREADS_2D_F64);
+        D == 3 ? (sizeof(T) == 4 ? OCA_PAIR_MAX_THREADS_3D : OCA_PAIR_MAX_THREADS_3D_F64)
+               : (sizeof(T) == 4 ? OCA_PAIR_MAX_THREADS_2D : OCA_PAIR_MAX_THREADS_2D_F64);
 };
 template <typename T, int D, int MODE, int SOLVER, int NR>
 __global__ void __launch_bounds__(PairBound<T, D>::threads, OCA_PAIR_MIN_BLOCKS) k_pair(PairArgs<T> a) {
@@ -794,11 +800,13 @@ cudaError_t launch_pose(const PoseArgs<T> &a, int maxQ, cudaStream_t st) {
     return cudaErrorInvalidValue;
 }
 
-int pair_max_warps(int dim, size_t es) {
+int pair_sm_warps(int dim, size_t es) {
     const int t = dim == 3 ? (es == 4 ? PairBound<float, 3>::threads : PairBound<double, 3>::threads)
                            : (es == 4 ? PairBound<float, 2>::threads : PairBound<double, 2>::threads);
     return t / 32;
 }
+
+int pair_max_warps(int dim, size_t es) { return dim == 3 ? 8 : pair_sm_warps(dim, es); }
 
 size_t pair_smem_bytes(int dim, size_t es, int W, int mode, int solver, int FR, int FO) {
     const int nstat = dim * (dim + 1) / 2 + dim + dim * dim;
