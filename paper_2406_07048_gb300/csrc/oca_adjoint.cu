@@ -8,20 +8,23 @@
 //   LQ    (s^{k+1}, u^{k+1}) = trajectory step linearised at (s^k, u^k)
 //   box   z^{k+1} = clip((s,u)^{k+1} + w^k),  w^{k+1} = w^k + (s,u)^{k+1} - z^{k+1}
 // and the reverse step k runs these backwards:
-//   k_adj_traj  box and LQ adjoints (the adjoint LQ shares the Riccati
-//               factorisation of the forward problem), then the chain rule
-//               through the linearisation point (second derivatives of the
-//               dynamics and of the part poses by dual numbers);
+//   launch_adj_traj  box and LQ adjoints (the adjoint LQ has the forward
+//               problem's matrices), then the chain rule through the
+//               linearisation point (second derivatives of the dynamics and
+//               of the part poses by dual numbers);
 //   k_adj_pair  per pair: statistics, pair QP (implicit differentiation of
 //               its optimality conditions in the (D+1)-dimensional dual form
 //               the forward solver uses) and head adjoints, reduced to pose
 //               adjoints per (part, t) and offset adjoints per obstacle face.
 // The pair QP is differentiated on its active set, which is locally constant
 // at strictly complementary solutions.
+#include <algorithm>
+
 #include "oca_common.cuh"
 #include "oca_dual.cuh"
 #include "oca_kernels.h"
 #include "oca_ric.cuh"
+#include "oca_ricprog.cuh"
 #include "oca_solvers.cuh"
 
 namespace oca {
@@ -121,7 +124,7 @@ __global__ void __launch_bounds__(32) k_adj_seed(AdjTrajArgs<T> a) {
 }
 
 // ============================================================================
-// reverse step k of the trajectory side (one warp per scenario)
+// reverse step k of the trajectory side, 12-state model (one warp per scenario)
 // ============================================================================
 template <typename T, typename F, int KIND>
 __global__ void __launch_bounds__(32) k_adj_traj(AdjTrajArgs<T> a) {
@@ -371,6 +374,392 @@ __global__ void __launch_bounds__(32) k_adj_traj(AdjTrajArgs<T> a) {
         }
         if (t < N)
             for (int i = 0; i < NU; ++i) a.ub[(long long)(sm.ctrl0 + t) * NU + i] = ubk[i];
+    }
+}
+
+// ============================================================================
+// reverse step k of the trajectory side, 2-D models: four kernels instead of one warp
+// per scenario doing everything (the LQ solve is the forward step's k_traj_lq).
+//   k_adj_pre      pose adjoints, box update, the stage records of the adjoint LQ
+//                  (lanes over t)
+//   k_traj_lq      its solution (xs, xu)
+//   k_adj_costate  costates of the forward and the adjoint solution (a warp each)
+//   k_adj_post     data adjoints and the chain rule into iterate k: a thread per
+//                  (step, direction), and the statistics' adjoints in closed form
+// Bound by FP64 issue in the chains.  256 trailer scenarios of horizon 50, a reverse
+// step: 358 us as one kernel, now 18 + 60 + 37 + 32 (gradient call 2.13 -> 1.78 ms).
+// ============================================================================
+constexpr int kAdjBlock = 96;
+
+template <typename T, typename F, int KIND>
+__global__ void __launch_bounds__(kAdjBlock) k_adj_pre(AdjTrajArgs<T> a) {
+    constexpr int NS = MDims<KIND>::NS, NU = MDims<KIND>::NU, D = MDims<KIND>::D, NROT = MDims<KIND>::NROT;
+    using Mp = RicMap<KIND>;
+    const int s = blockIdx.x, k = a.k;
+    if (k >= a.iters[s]) return;
+    const ScenMeta sm = a.meta[s];
+    const int N = sm.N;
+    const TapeView<T> &tp = a.tape;
+    const T *s_k = tp.s + (long long)k * tp.s_slot, *u_k = tp.u + (long long)k * tp.u_slot;
+    const T *s_k1 = tp.s + (long long)(k + 1) * tp.s_slot, *u_k1 = tp.u + (long long)(k + 1) * tp.u_slot;
+    const T *zs_k = tp.box + (long long)k * tp.box_slot;
+    const T *ws_k = zs_k + tp.n_states * NS, *zu_k = ws_k + tp.n_states * NS, *wu_k = zu_k + tp.n_ctrls * NU;
+    F *scr = reinterpret_cast<F *>(a.scratch) + a.scratch0[s];
+    StageParams<T> sp;
+    sp.model = a.model;
+    sp.g = a.g;
+    sp.sigma = a.sigma;
+    sp.rho_box = a.rho_box;
+    sp.damp = a.damp;
+    sp.s_ref = a.s_ref;
+    sp.Qtot = a.Qtot;
+    StageSrc<T> src;
+    src.s = s_k;
+    src.u = u_k;
+    src.zs = zs_k;
+    src.ws = ws_k;
+    src.zu = zu_k;
+    src.wu = wu_k;
+    src.stats = tp.stats + (long long)k * tp.stats_slot;
+    struct Sink {
+        F *r;
+        F x[NS], g[NS];  // s^{k+1}_t; Q x + q
+        __device__ void A(int i, int j, T v) {
+            const int e = RicSparse<KIND>::a_slot(i, j);
+            if (e >= 0) r[Mp::rA + e] = F(v);
+        }
+        __device__ void B(int i, int j, T v) {
+            const int e = RicSparse<KIND>::b_slot(i, j);
+            if (e >= 0) r[Mp::rB + e] = F(v);
+        }
+        __device__ void c(int, T) {}
+        __device__ void u(int, T) {}
+        __device__ void Q(int i, int j, T v) {
+            if (i <= j) r[Mp::rQ + Mp::sym(i, j)] = F(v);
+            g[i] = j == 0 ? F(v) * x[0] : fma(F(v), x[j], g[i]);
+        }
+        __device__ void q(int i, T v) { g[i] += F(v); }
+    };
+    for (int t = threadIdx.x; t <= N; t += blockDim.x) {
+        // pose adjoints of s^{k+1} (pair side of iteration k+1), then the box update of
+        // iteration k (z = clip(x + w), w += x - z)
+        const long long ks = (long long)(sm.state0 + t) * NS, ku = (long long)(sm.ctrl0 + t) * NU;
+        T st[NS], sb[NS], ub[NU];
+#pragma unroll
+        for (int i = 0; i < NS; ++i) {
+            st[i] = s_k1[ks + i];
+            sb[i] = a.sb[ks + i];
+        }
+        if (t >= 1) {
+            T acc[NS];
+#pragma unroll
+            for (int i = 0; i < NS; ++i) acc[i] = T(0);
+            for (int part = 0; part < sm.NP; ++part) {
+                const int gp = sm.part0 + part;
+                T off[D], rho[D], R[D * D], drho[D * NS], dR[NROT][D * D];
+                int ridx[NROT];
+#pragma unroll
+                for (int i = 0; i < D; ++i) off[i] = a.g.part_off[gp * D + i];
+                part_pose<T, KIND>(a.model, a.g.part_link[gp], off, st, rho, R, drho, dR, ridx);
+                const long long col = sm.qbeg + part * N + (t - 1);
+#pragma unroll
+                for (int i = 0; i < D; ++i) {
+                    const T rb = a.poseb[(long long)i * a.Qtot + col];
+#pragma unroll
+                    for (int e = 0; e < NS; ++e) acc[e] += rb * drho[i * NS + e];
+                }
+                T v = T(0);
+#pragma unroll
+                for (int i = 0; i < D * D; ++i) v += a.poseb[(long long)(D + i) * a.Qtot + col] * dR[0][i];
+#pragma unroll
+                for (int e = 0; e < NS; ++e)
+                    if (e == ridx[0]) acc[e] += v;
+            }
+#pragma unroll
+            for (int i = 0; i < NS; ++i) sb[i] += acc[i];
+        }
+        const bool box = a.rho_box > T(0);
+        auto unbox = [&](T x, T lo, T hi, T w, T *zb, T *wb, T &xb) {
+            const T wbar = *wb, zp = *zb - wbar, v = x + w;
+            T xa = xb + wbar, wn = wbar;
+            if (v > lo && v < hi) {
+                xa += zp;
+                wn += zp;
+            }
+            xb = xa;
+            *wb = wn;
+            *zb = T(0);
+        };
+        if (t >= 1 && box)
+#pragma unroll
+            for (int i = 0; i < NS; ++i)
+                if (bounded(a.model.s_lo[i], a.model.s_hi[i]))
+                    unbox(st[i], a.model.s_lo[i], a.model.s_hi[i], ws_k[ks + i], a.zsb + ks + i, a.wsb + ks + i, sb[i]);
+        F *rec = scr + Mp::rec(t);
+        if (t < N) {
+#pragma unroll
+            for (int i = 0; i < NU; ++i) {
+                ub[i] = a.ub[ku + i];
+                if (box && bounded(a.model.u_lo[i], a.model.u_hi[i]))
+                    unbox(u_k1[ku + i], a.model.u_lo[i], a.model.u_hi[i], wu_k[ku + i], a.zub + ku + i, a.wub + ku + i, ub[i]);
+                rec[Mp::rr + i] = -F(ub[i]);
+            }
+#pragma unroll
+            for (int i = 0; i < NS; ++i) rec[Mp::rc + i] = F(0);
+        }
+        // the adjoint LQ has the forward one's Q, Ru, A, B, linear terms -sbar, -ubar, c = 0
+        // and s_0 = 0; sbar of the fixed initial state passes to the initial-state adjoint
+#pragma unroll
+        for (int i = 0; i < NS; ++i) {
+            rec[Mp::rq + i] = t >= 1 ? -F(sb[i]) : F(0);
+            if (t == 0) {
+                a.gs0[(long long)s * NS + i] += double(sb[i]);
+                scr[Mp::s0(N) + i] = F(0);
+            }
+        }
+        Sink out;
+        out.r = rec;
+#pragma unroll
+        for (int i = 0; i < NS; ++i) out.x[i] = F(st[i]);
+        assemble_terms<T, KIND>(sp, src, sm, t, out);
+#pragma unroll
+        for (int i = 0; i < NS; ++i) scr[Mp::adj(N, 0, t) + i] = out.g[i];
+    }
+}
+
+// Costates pi_t = g_t + A_t^T pi_{t+1}, g_t = Q_t x_t + q_t, of the forward solution
+// (g from k_adj_pre; warp 0) and of the adjoint one (g formed here first; warp 1).
+// Lane i owns pi_i; the steps' coefficients are on their way four steps ahead.
+template <typename F, int KIND>
+__global__ void __launch_bounds__(64) k_adj_costate(const ScenMeta *meta, const int *iters, int k, void *scratch,
+                                                    const long long *scratch0) {
+    constexpr int NS = MDims<KIND>::NS, AHEAD = 4;
+    using Mp = RicMap<KIND>;
+    const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, which = tid >> 5;
+    if (k >= iters[s]) return;
+    const int N = meta[s].N;
+    F *scr = reinterpret_cast<F *>(scratch) + scratch0[s];
+    for (int e = tid; e < N * NS; e += 64) {
+        const int t = 1 + e / NS, i = e % NS;
+        const F *rec = scr + Mp::rec(t), *x = scr + Mp::sol(N, t - 1);  // xs_t
+        F acc = rec[Mp::rq + i];
+#pragma unroll
+        for (int j = 0; j < NS; ++j) acc = fma(rec[Mp::rQ + Mp::sym(i, j)], x[j], acc);
+        scr[Mp::adj(N, 1, t) + i] = acc;
+    }
+    __syncthreads();
+    const int i = lane < NS ? lane : 0;
+    int slot[NS];  // where A[l][i] is read: record entry, or -1: 0, -2: 1
+#pragma unroll
+    for (int l = 0; l < NS; ++l) {
+        const int e = RicSparse<KIND>::a_slot(l, i);
+        slot[l] = e >= 0 ? e : l == i ? -2 : -1;
+    }
+    F col[AHEAD][NS], g[AHEAD];
+    auto fetch = [&](int t, F (&c)[NS], F &gt) {  // step t: pi_t from pi_{t+1}
+        const int tc = max(t, 1);
+        const F *rec = scr + Mp::rec(min(tc, N - 1));  // t = N: pi_{N+1} = 0
+#pragma unroll
+        for (int l = 0; l < NS; ++l) c[l] = slot[l] >= 0 ? rec[Mp::rA + slot[l]] : slot[l] == -2 ? F(1) : F(0);
+        gt = scr[Mp::adj(N, which, tc) + i];
+    };
+    F pi = F(0);
+#pragma unroll
+    for (int d = 0; d < AHEAD; ++d) fetch(N - d, col[d], g[d]);
+    for (int t0 = N; t0 >= 1; t0 -= AHEAD) {
+#pragma unroll
+        for (int d = 0; d < AHEAD; ++d) {
+            const int t = t0 - d;
+            F v = g[d];
+#pragma unroll
+            for (int l = 0; l < NS; ++l) v = fma(col[d][l], __shfl_sync(0xffffffffu, pi, l), v);
+            if (t >= 1) {
+                pi = v;
+                if (lane < NS) scr[Mp::adj(N, 2 + which, t) + lane] = v;
+            }
+            fetch(t - AHEAD, col[d], g[d]);
+        }
+    }
+}
+
+// Per step t, with (s, u) = (s^{k+1}, u^{k+1}), (xs, xu) the adjoint solution, pf, pa the
+// costates and the linearisation point (s^k, u^k):
+//   At = Abar - cbar s_k^T, Bt = Bbar - cbar u_k^T (Abar = -(pa s^T + pf xs^T),
+//   Bbar = -(pa u^T + pf xu^T), cbar = -pa), qb = -xs, G = -xs s^T - qb s_k^T,
+// then a thread per (step, direction e) of (s^k, u^k): d/de of At : fs + Bt : fu (dual
+// numbers), the damping and box terms, and for e in s^k the Gauss-Newton terms of every
+// part; and a thread per (step, part) for the statistics' adjoints, in closed form since
+// the terms are linear in W, Wc and E.
+constexpr int kPostSteps = 32, kPostThreads = 256;
+template <typename T, typename F, int KIND>
+__global__ void __launch_bounds__(kPostThreads) k_adj_post(AdjTrajArgs<T> a) {
+    constexpr int NS = MDims<KIND>::NS, NU = MDims<KIND>::NU, D = MDims<KIND>::D, NROT = MDims<KIND>::NROT, NZ = NS + NU;
+    constexpr int NW = StatDims<D>::NW, NSTAT = StatDims<D>::NSTAT;
+    constexpr int oB = NS * NS, oG = oB + NS * NU, oq = oG + NS * NS, W = (oq + NS) | 1;
+    using Mp = RicMap<KIND>;
+    __shared__ T mat[kPostSteps * W];  // At, Bt, G, qb of each step
+    const int s = blockIdx.x, tid = threadIdx.x, k = a.k;
+    if (k >= a.iters[s]) return;
+    const ScenMeta sm = a.meta[s];
+    const int N = sm.N, t0 = blockIdx.y * kPostSteps, nt = min(kPostSteps, N + 1 - t0);
+    if (nt <= 0) return;
+    const TapeView<T> &tp = a.tape;
+    const T *s_k = tp.s + (long long)k * tp.s_slot, *u_k = tp.u + (long long)k * tp.u_slot;
+    const T *s_k1 = tp.s + (long long)(k + 1) * tp.s_slot, *u_k1 = tp.u + (long long)(k + 1) * tp.u_slot;
+    const T *stats_k = tp.stats + (long long)k * tp.stats_slot;
+    const F *scr = reinterpret_cast<const F *>(a.scratch) + a.scratch0[s];
+    // xs_t, xu_t: rows [s_{t+1}, u_t] of the solution
+    auto xs = [&](int t, int i) -> F { return t >= 1 ? scr[Mp::sol(N, t - 1) + i] : F(0); };
+    for (int e = tid; e < nt * NS; e += kPostThreads) {
+        // row i of the matrices of step t
+        const int t = t0 + e / NS, i = e % NS;
+        T *m = mat + (t - t0) * W;
+        const long long ks = (long long)(sm.state0 + t) * NS, ku = (long long)(sm.ctrl0 + t) * NU;
+        if (t < N) {
+            const F pf1 = scr[Mp::adj(N, 2, t + 1) + i], pa1 = scr[Mp::adj(N, 3, t + 1) + i], cb = -pa1;
+#pragma unroll
+            for (int j = 0; j < NS; ++j)
+                m[i * NS + j] = T(-(pa1 * F(s_k1[ks + j]) + pf1 * xs(t, j)) - cb * F(s_k[ks + j]));
+#pragma unroll
+            for (int j = 0; j < NU; ++j)
+                m[oB + i * NU + j] = T(-(pa1 * F(u_k1[ku + j]) + pf1 * scr[Mp::sol(N, t) + NS + j]) - cb * F(u_k[ku + j]));
+        }
+        const F xh = xs(t, i);
+        const T qb = T(-xh);
+        m[oq + i] = qb;
+#pragma unroll
+        for (int j = 0; j < NS; ++j) m[oG + i * NS + j] = T(-xh * F(s_k1[ks + j])) - qb * s_k[ks + j];
+    }
+    __syncthreads();
+    const T rho_b = a.rho_box, damp = a.damp;
+    const int n_dir = nt * NZ, n_item = n_dir + nt * sm.NP;
+    for (int item = tid; item < n_item; item += kPostThreads) {
+        const bool dir = item < n_dir;
+        // directions of one kind side by side: the lanes of a warp share a path
+        const int t = t0 + (dir ? item % nt : (item - n_dir) % nt);
+        const T *m = mat + (t - t0) * W, *qb = m + oq, *G = m + oG;
+        const long long ks = (long long)(sm.state0 + t) * NS, ku = (long long)(sm.ctrl0 + t) * NU;
+        T st[NS];
+#pragma unroll
+        for (int i = 0; i < NS; ++i) st[i] = s_k[ks + i];
+        if (!dir) {
+            const int part = (item - n_dir) / nt;
+            if (t == 0) continue;
+            const int gp = sm.part0 + part;
+            T off[D], rho[D], R[D * D], drho[D * NS], dR[NROT][D * D];
+            int ridx[NROT];
+#pragma unroll
+            for (int i = 0; i < D; ++i) off[i] = a.g.part_off[gp * D + i];
+            part_pose<T, KIND>(a.model, a.g.part_link[gp], off, st, rho, R, drho, dR, ridx);
+            T v[D], qa = T(0), gaa = T(0), Wb[D][D];
+#pragma unroll
+            for (int i = 0; i < D; ++i) v[i] = T(0);
+#pragma unroll
+            for (int e = 0; e < NS; ++e) {
+#pragma unroll
+                for (int i = 0; i < D; ++i) v[i] += qb[e] * drho[i * NS + e];
+                if (e == ridx[0]) {
+                    qa = qb[e];
+                    gaa = G[e * NS + e];
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < D; ++i)
+#pragma unroll
+                for (int j = 0; j < D; ++j) {
+                    T acc = v[i] * rho[j];
+#pragma unroll
+                    for (int e = 0; e < NS; ++e) {
+                        T gd = T(0);
+#pragma unroll
+                        for (int f = 0; f < NS; ++f) gd += G[e * NS + f] * drho[j * NS + f];
+                        acc += drho[i * NS + e] * gd;
+                    }
+#pragma unroll
+                    for (int l = 0; l < D; ++l) acc += dR[0][i * D + l] * (gaa * dR[0][j * D + l] + qa * R[j * D + l]);
+                    Wb[i][j] = acc;
+                }
+            const long long col = sm.qbeg + part * N + (t - 1);
+            int kk = 0;
+#pragma unroll
+            for (int i = 0; i < D; ++i)
+#pragma unroll
+                for (int j = 0; j <= i; ++j, ++kk)
+                    a.statsb[(long long)kk * a.Qtot + col] = a.sigma * (i == j ? Wb[i][i] : Wb[i][j] + Wb[j][i]);
+#pragma unroll
+            for (int i = 0; i < D; ++i) a.statsb[(long long)(NW + i) * a.Qtot + col] = -a.sigma * v[i];
+#pragma unroll
+            for (int i = 0; i < D * D; ++i) a.statsb[(long long)(NW + D + i) * a.Qtot + col] = a.sigma * qa * dR[0][i];
+            continue;
+        }
+        const int e = item / nt;
+        T out = T(0);
+        if (t < N) {
+            const DevModel<Dual<T>> dm = dual_model(a.model);
+            Dual<T> sd[NS], ud[NU], f[NS], fs[NS * NS], fu[NS * NU];
+#pragma unroll
+            for (int i = 0; i < NS; ++i) sd[i] = Dual<T>(st[i], i == e ? T(1) : T(0));
+#pragma unroll
+            for (int i = 0; i < NU; ++i) ud[i] = Dual<T>(u_k[ku + i], i + NS == e ? T(1) : T(0));
+            dynamics<Dual<T>, KIND>(dm, sd, ud, f, fs, fu);
+            T acc = T(0);
+#pragma unroll
+            for (int i = 0; i < NS * NS; ++i) acc += m[i] * fs[i].d;
+#pragma unroll
+            for (int i = 0; i < NS * NU; ++i) acc += m[oB + i] * fu[i].d;
+            out += a.model.dt * acc;
+        }
+        if (e >= NS) {
+            if (t == N) continue;
+            const int i = e - NS;
+            const T rb = T(-scr[Mp::sol(N, t) + NS + i]);
+            out -= damp * rb;
+            if (rho_b > T(0) && bounded(a.model.u_lo[i], a.model.u_hi[i])) {
+                a.zub[ku + i] = -rho_b * rb;
+                a.wub[ku + i] += rho_b * rb;
+            }
+            a.ub[ku + i] = out;
+            continue;
+        }
+        if (t == 0) {
+            // s_0 enters the first dynamics constraint as data: -A_0^T pa_1
+            const F *rec = scr + Mp::rec(0);
+            F acc = F(0);
+#pragma unroll
+            for (int i = 0; i < NS; ++i) {
+                const int sl = RicSparse<KIND>::a_slot(i, e);
+                const F A0 = sl >= 0 ? rec[Mp::rA + sl] : i == e ? F(1) : F(0);
+                acc -= A0 * scr[Mp::adj(N, 3, 1) + i];
+            }
+            out += T(acc);
+            a.gs0[(long long)s * NS + e] += double(out);
+            a.sb[ks + e] = T(0);
+            continue;
+        }
+        const T qe = qb[e];
+        out -= damp * qe;
+        if (rho_b > T(0) && bounded(a.model.s_lo[e], a.model.s_hi[e])) {
+            a.zsb[ks + e] = -rho_b * qe;
+            a.wsb[ks + e] += rho_b * qe;
+        }
+        for (int part = 0; part < sm.NP; ++part) {
+            const int gp = sm.part0 + part;
+            const long long col = sm.qbeg + part * N + (t - 1);
+            const DevModel<Dual<T>> dm = dual_model(a.model);
+            Dual<T> offd[D], sd[NS], stat[NSTAT], Hs[NS * NS], g[NS];
+#pragma unroll
+            for (int i = 0; i < D; ++i) offd[i] = Dual<T>(a.g.part_off[gp * D + i]);
+#pragma unroll
+            for (int i = 0; i < NSTAT; ++i) stat[i] = Dual<T>(stats_k[(long long)i * a.Qtot + col]);
+#pragma unroll
+            for (int i = 0; i < NS; ++i) sd[i] = Dual<T>(st[i], i == e ? T(1) : T(0));
+            gn_part<Dual<T>, KIND>(dm, a.g.part_link[gp], offd, sd, stat, stat + NW, stat + NW + D, Hs, g);
+            T acc = T(0);
+            for (int i = 0; i < NS * NS; ++i) acc += G[i] * Hs[i].d;
+            for (int i = 0; i < NS; ++i) acc += qb[i] * (g[i].d - Hs[i * NS + e].v);
+            out += a.sigma * acc;
+        }
+        a.sb[ks + e] = out;
     }
 }
 
@@ -852,11 +1241,24 @@ cudaError_t launch_adj_seed(const AdjTrajArgs<T> &a, int n_scen, cudaStream_t st
     return cudaGetLastError();
 }
 
+template <typename T, int KIND>
+cudaError_t launch_adj_traj_2d(const AdjTrajArgs<T> &a, int n_scen, int *lq_ok, const int *order, int max_n, int n_sm,
+                               cudaStream_t st) {
+    const int steps = std::min(kAdjBlock, (max_n + 1 + 31) / 32 * 32);
+    k_adj_pre<T, double, KIND><<<n_scen, steps, 0, st>>>(a);
+    cudaError_t e = launch_adj_lq<T>(a, n_scen, lq_ok, order, n_sm, st);
+    if (e != cudaSuccess) return e;
+    k_adj_costate<double, KIND><<<n_scen, 64, 0, st>>>(a.meta, a.iters, a.k, a.scratch, a.scratch0);
+    k_adj_post<T, double, KIND><<<dim3(n_scen, (max_n + kPostSteps) / kPostSteps), kPostThreads, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
 template <typename T>
-cudaError_t launch_adj_traj(const AdjTrajArgs<T> &a, int n_scen, cudaStream_t st) {
+cudaError_t launch_adj_traj(const AdjTrajArgs<T> &a, int n_scen, int *lq_ok, const int *order, int max_n, int n_sm,
+                            cudaStream_t st) {
     switch (a.model.kind) {
-        case 0: k_adj_traj<T, double, 0><<<n_scen, 32, 0, st>>>(a); break;
-        case 1: k_adj_traj<T, double, 1><<<n_scen, 32, 0, st>>>(a); break;
+        case 0: return launch_adj_traj_2d<T, 0>(a, n_scen, lq_ok, order, max_n, n_sm, st);
+        case 1: return launch_adj_traj_2d<T, 1>(a, n_scen, lq_ok, order, max_n, n_sm, st);
         case 2: k_adj_traj<T, double, 2><<<n_scen, 32, 0, st>>>(a); break;
         default: return cudaErrorInvalidValue;
     }
@@ -910,8 +1312,8 @@ cudaError_t launch_adj_finish(const double *gd, const T *obs_C, const int *obs_n
 
 template cudaError_t launch_adj_seed<float>(const AdjTrajArgs<float> &, int, cudaStream_t);
 template cudaError_t launch_adj_seed<double>(const AdjTrajArgs<double> &, int, cudaStream_t);
-template cudaError_t launch_adj_traj<float>(const AdjTrajArgs<float> &, int, cudaStream_t);
-template cudaError_t launch_adj_traj<double>(const AdjTrajArgs<double> &, int, cudaStream_t);
+template cudaError_t launch_adj_traj<float>(const AdjTrajArgs<float> &, int, int *, const int *, int, int, cudaStream_t);
+template cudaError_t launch_adj_traj<double>(const AdjTrajArgs<double> &, int, int *, const int *, int, int, cudaStream_t);
 template cudaError_t launch_adj_pair<float>(const AdjPairArgs<float> &, int, int, int, cudaStream_t);
 template cudaError_t launch_adj_pair<double>(const AdjPairArgs<double> &, int, int, int, cudaStream_t);
 template cudaError_t launch_adj_alpha<float>(const AdjAlphaArgs<float> &, int, int, int, const int *, const float *,

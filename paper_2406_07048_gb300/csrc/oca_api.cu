@@ -801,7 +801,7 @@ oca_status backward_impl(oca_scene *sc, const oca_model *m, const oca_admm_param
     ap.gd = gd;
     for (int k = K - 1; k >= 0; --k) {
         ta.k = k;
-        OCA_CK(launch_adj_traj<T>(ta, sc->S, st));
+        OCA_CK(launch_adj_traj<T>(ta, sc->S, sc->d_lq_ok, sc->d_order, sc->maxN, sc->ctx->n_sm, st));
         pa.states = tp + TL.s + (long long)k * tv.s_slot;
         OCA_CK(launch_pose<T>(pa, sc->maxQ, st));
         ap.k = k;

@@ -35,8 +35,13 @@ long long riccati_scratch_elems(int kind, int N);
 // adjoint of a taped ADMM solve (oca_adjoint.cu)
 template <typename T>
 cudaError_t launch_adj_seed(const AdjTrajArgs<T> &a, int n_scen, cudaStream_t st);
+// trajectory side of a reverse step; lq_ok, order, max_n, n_sm as launch_riccati's
 template <typename T>
-cudaError_t launch_adj_traj(const AdjTrajArgs<T> &a, int n_scen, cudaStream_t st);
+cudaError_t launch_adj_traj(const AdjTrajArgs<T> &a, int n_scen, int *lq_ok, const int *order, int max_n, int n_sm,
+                            cudaStream_t st);
+// its LQ problem (2-D models; oca_riccati.cu)
+template <typename T>
+cudaError_t launch_adj_lq(const AdjTrajArgs<T> &a, int n_scen, int *lq_ok, const int *order, int n_sm, cudaStream_t st);
 template <typename T>
 cudaError_t launch_adj_pair(const AdjPairArgs<T> &a, int dim, int n_tiles, int W, cudaStream_t st);
 template <typename T>

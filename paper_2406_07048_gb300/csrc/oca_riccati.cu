@@ -28,9 +28,9 @@ namespace oca {
 
 long long riccati_scratch_elems(int kind, int N) {
     switch (kind) {
-        // the forward step's packed records and the adjoint's dense layout share the block
-        case 0: return std::max(RicLayout<4, 2>::size(N), RicMap<0>::size(N));
-        case 1: return std::max(RicLayout<5, 2>::size(N), RicMap<1>::size(N));
+        // the forward step's and the adjoint's share the block (12 states: the adjoint's is dense)
+        case 0: return RicMap<0>::adj_size(N);
+        case 1: return RicMap<1>::adj_size(N);
         default: return std::max(RicLayout<12, 4>::size(N), RicMap<2>::size(N));
     }
 }
@@ -560,12 +560,16 @@ struct LqArgs2 {
     const ScenMeta *meta;
     const int *order;        // scenarios by descending horizon
     int n_scen;
-    const int *scen_status;
+    const int *scen_status;  // forward: scenarios with kActive are solved
+    const int *iters;        // adjoint (not null): scenarios with k < iters
+    int k;
     void *scratch;
     const long long *scratch0;
     F dt, ru[4];
     int *ok;                 // [S] out: factorisation and sweep finite and positive definite
-    int *iter;               // advanced by one
+    int *iter;               // advanced by one (null: none)
+
+    __device__ __forceinline__ bool active(int s) const { return iters ? k < iters[s] : scen_status[s] == kActive; }
 };
 
 // One CTA per SM, two warps per scheduler.  A group of 32 / L scenarios (neighbours
@@ -586,7 +590,7 @@ __global__ void __launch_bounds__(32 * kLqWarps) k_traj_lq(LqArgs2<F> a) {
     constexpr int PR = (REC + L - 1) / L, PO = (OUT + L - 1) / L, KE = NU * (NS + 1), PK = (KE + L - 1) / L;
     __shared__ F region[kLqWarps][G][Mp::SIZE];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane / L, li = lane % L;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *a.iter += 1;
+    if (a.iter && blockIdx.x == 0 && threadIdx.x == 0) *a.iter += 1;
     const int n_group = (a.n_scen + G - 1) / G, K = 4 * gridDim.x, slot = (warp & 3) * gridDim.x + blockIdx.x;
     F *sm = region[warp][g];
 
@@ -610,7 +614,7 @@ __global__ void __launch_bounds__(32 * kLqWarps) k_traj_lq(LqArgs2<F> a) {
     const int group = round & 1 ? (round + 1) * K - 1 - slot : round * K + slot;
     const int at = group * G + g;
     const int s = group < n_group && at < a.n_scen ? a.order[at] : -1;
-    const bool live = s >= 0 && a.scen_status[s] == kActive;
+    const bool live = s >= 0 && a.active(s);
     if (!__any_sync(0xffffffffu, live)) continue;
     const int N = live ? a.meta[s].N : 0;
     int Nm = N;
@@ -734,8 +738,8 @@ __global__ void __launch_bounds__(128) k_traj_lq4(LqArgs2<F> a) {
     constexpr int PR = (REC + NT - 1) / NT, PO = (OUT + NT - 1) / NT;
     __shared__ F sm[Mp::SIZE];
     const int tid = threadIdx.x, lane = tid & 31, s = a.order[blockIdx.x];
-    if (blockIdx.x == 0 && tid == 0) *a.iter += 1;
-    if (a.scen_status[s] != kActive) return;
+    if (a.iter && blockIdx.x == 0 && tid == 0) *a.iter += 1;
+    if (!a.active(s)) return;
     const int N = a.meta[s].N;
     F *scr = reinterpret_cast<F *>(a.scratch) + a.scratch0[s];
     typename LqSlotsOf<F, std::remove_cv_t<decltype(kRicTab<2, NT, 0>)>>::type prod_y;
@@ -902,6 +906,26 @@ __global__ void __launch_bounds__(kTrajBlock) k_traj_apply(RicArgs<T> a, const i
 // no more scenarios than schedulers (4 per SM) every one has its own warp and 32
 // lanes are the shorter chain (256 scenarios of horizon 50: 2,290 cycles per stage).
 // 2,048 scenarios: 138 us with 16 lanes, 174 with 32.
+template <typename F, int KIND>
+void launch_lq_solve(const LqArgs2<F> &l, int n_sm, cudaStream_t st) {
+    if constexpr (KIND == 2) {
+        k_traj_lq4<F><<<l.n_scen, 128, 0, st>>>(l);
+    } else {
+        const bool one = l.n_scen <= 4 * n_sm;
+        const int groups = one ? l.n_scen : (l.n_scen + 1) / 2, ctas = std::min(n_sm, groups);
+        if (one) k_traj_lq<F, KIND, 32><<<ctas, 32 * kLqWarps, 0, st>>>(l);
+        else k_traj_lq<F, KIND, 16><<<ctas, 32 * kLqWarps, 0, st>>>(l);
+    }
+}
+
+// dt and the diagonal of Ru
+template <typename T, typename F>
+void lq_constants(LqArgs2<F> &l, const DevModel<T> &m, T damp, T rho_box, int nu) {
+    l.dt = F(m.dt);
+    for (int i = 0; i < nu; ++i)
+        l.ru[i] = F(2) * F(m.Qu[i]) + F(damp) + (m.u_lo[i] > T(-1e29) || m.u_hi[i] < T(1e29) ? F(rho_box) : F(0));
+}
+
 template <typename T, typename F, int KIND>
 cudaError_t launch_traj(const RicArgs<T> &a, int *lq_ok, const int *order, int max_n, int n_sm, cudaStream_t st) {
     LqArgs2<F> l;
@@ -909,23 +933,16 @@ cudaError_t launch_traj(const RicArgs<T> &a, int *lq_ok, const int *order, int m
     l.order = order;
     l.n_scen = a.n_scen;
     l.scen_status = a.scen_status;
+    l.iters = nullptr;
+    l.k = 0;
     l.scratch = a.scratch;
     l.scratch0 = a.scratch0;
-    l.dt = F(a.model.dt);
-    for (int i = 0; i < MDims<KIND>::NU; ++i)
-        l.ru[i] = F(2) * F(a.model.Qu[i]) + F(a.damp) +
-                  (a.model.u_lo[i] > T(-1e29) || a.model.u_hi[i] < T(1e29) ? F(a.rho_box) : F(0));
+    lq_constants<T, F>(l, a.model, a.damp, a.rho_box, MDims<KIND>::NU);
     l.ok = lq_ok;
     l.iter = a.iter;
     const int steps = std::min(kTrajBlock, (max_n + 1 + 31) / 32 * 32);
     k_traj_stage<T, F, KIND><<<a.n_scen, steps, sizeof(F) * steps * traj_rec_stride<F, KIND>(), st>>>(a);
-    if constexpr (KIND == 2) {
-        k_traj_lq4<F><<<a.n_scen, 128, 0, st>>>(l);
-    } else {
-        const int one = a.n_scen <= 4 * n_sm, groups = one ? a.n_scen : (a.n_scen + 1) / 2, ctas = std::min(n_sm, groups);
-        if (one) k_traj_lq<F, KIND, 32><<<ctas, 32 * kLqWarps, 0, st>>>(l);
-        else k_traj_lq<F, KIND, 16><<<ctas, 32 * kLqWarps, 0, st>>>(l);
-    }
+    launch_lq_solve<F, KIND>(l, n_sm, st);
     k_traj_apply<T, F, KIND><<<a.n_scen, steps, 0, st>>>(a, lq_ok);
     return cudaGetLastError();
 }
@@ -939,6 +956,28 @@ cudaError_t launch_riccati_f(const RicArgs<T> &a, int *lq_ok, const int *order, 
     }
     return cudaErrorInvalidValue;
 }
+
+template <typename T>
+cudaError_t launch_adj_lq(const AdjTrajArgs<T> &a, int n_scen, int *lq_ok, const int *order, int n_sm, cudaStream_t st) {
+    LqArgs2<double> l;
+    l.meta = a.meta;
+    l.order = order;
+    l.n_scen = n_scen;
+    l.scen_status = nullptr;
+    l.iters = a.iters;
+    l.k = a.k;
+    l.scratch = a.scratch;
+    l.scratch0 = a.scratch0;
+    lq_constants<T, double>(l, a.model, a.damp, a.rho_box, 2);
+    l.ok = lq_ok;
+    l.iter = nullptr;
+    if (a.model.kind == 0) launch_lq_solve<double, 0>(l, n_sm, st);
+    else if (a.model.kind == 1) launch_lq_solve<double, 1>(l, n_sm, st);
+    else return cudaErrorInvalidValue;
+    return cudaGetLastError();
+}
+template cudaError_t launch_adj_lq<float>(const AdjTrajArgs<float> &, int, int *, const int *, int, cudaStream_t);
+template cudaError_t launch_adj_lq<double>(const AdjTrajArgs<double> &, int, int *, const int *, int, cudaStream_t);
 
 template <typename T>
 cudaError_t launch_riccati(const RicArgs<T> &a, bool f32, int *lq_ok, const int *order, int max_n, int n_sm, cudaStream_t st) {

@@ -116,6 +116,12 @@ struct RicMap {
     __host__ __device__ static long long s0(int N) { return out(N, N); }
     __host__ __device__ static long long sol(int N, int t) { return s0(N) + NS + (long long)t * NZ; }
     __host__ __device__ static long long size(int N) { return sol(N, N); }
+    // behind them, the adjoint's vectors of t = 0..N: which = 0, 1 the sources Q x + q of
+    // the forward and adjoint costates, 2, 3 the costates
+    __host__ __device__ static long long adj(int N, int which, int t) {
+        return size(N) + ((long long)which * (N + 1) + t) * NS;
+    }
+    __host__ __device__ static long long adj_size(int N) { return adj(N, 4, 0); }
     static constexpr int sym(int i, int j) { return i <= j ? i * NS - i * (i - 1) / 2 + (j - i) : sym(j, i); }
 };
 

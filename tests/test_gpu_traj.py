@@ -54,3 +54,54 @@ def test_trajectory_split_matches_oracle(B, ora, n_scen):
         c, d = int(sc.ctrl_begin[s]), int(sc.ctrl_begin[s + 1])
         for got, want in ((s_g[a:b], ref["s"][a:b]), (u_g[c:d], ref["u"][c:d])):
             assert np.abs(got - want).max() <= 1e-9 * (1.0 + np.abs(want).max()), (s, horizons[s])
+
+
+@pytest.mark.parametrize("extra", [0, 600])
+def test_adjoint_split_matches_finite_differences(B, ora, extra):
+    """Reverse steps over horizons around a block of steps (32 in the chain rule, 96 in
+    the assembly) and over counts that take one and two scenarios per warp: gradients
+    by the initial state and by the first obstacle's translation, against central
+    differences of the oracle's costs per scenario (step 1e-4: the rounding of the
+    costs, divided by the step, falls below the bound, which allows for
+    two FP64 costs with a hundredfold growth over the steps and a step of 1e-6:
+    1e-8 of the cost); 1e-4 relative is the bound of the other gradient tests."""
+    import dataclasses
+
+    horizons = [1, 2, 5, 31, 32, 33, 63, 64, 95, 96, 97] + [1] * extra
+    sc, K, h = _bicycles(horizons), 3, 1e-4
+    kw = dict(sigma=300.0, eps_pri=0.0, eps_dual=0.0, prox=0.1, rho_box=100.0, damp=100.0)
+    row0 = np.concatenate([[0], np.cumsum([n + 1 for n in horizons])[:-1]])
+    obs0 = np.asarray(sc.obs_begin)[:-1]
+
+    def differences(change):
+        costs = [ora.admm_batch(change(e), max_iter=K, **kw)["cost"] for e in (h, -h)]
+        return (costs[0] - costs[1]) / (2 * h), np.abs(costs[0])
+
+    def state(i):
+        def change(e):
+            s = sc.s_init.copy()
+            s[row0, i] += e
+            return dataclasses.replace(sc, s_init=s)
+        return change
+
+    def shift(i):
+        def change(e):
+            d = sc.obs_d.copy()
+            d[obs0] += e * sc.obs_C[obs0][:, :, i]
+            return dataclasses.replace(sc, obs_d=d)
+        return change
+
+    ctx = B.Context(0)
+    ds = B.DeviceScene(ctx, sc, torch.float64)
+    pb = B.Problem(ds)
+    tape = B.new_tape(ds, K)
+    rep = B.admm_solve(ds, pb.s_ref, pb.s, pb.u, pb.y, pb.zeta, pb.xi, tape=tape, max_iter=K, **kw)
+    g = B.admm_backward(ds, pb.s_ref, tape, rep["iters"], torch.ones(sc.n_scen, dtype=torch.float64, device=ds.device),
+                        max_iter=K, **{k: kw[k] for k in ("sigma", "prox", "rho_box", "damp")})
+    g = {k: v.cpu().numpy() for k, v in g.items()}
+    for i in range(sc.model.ns):
+        fd, cost = differences(state(i))
+        assert np.all(np.abs(g["state0"][:, i] - fd) <= 1e-4 * np.abs(fd) + 1e-8 * cost + 1e-8), i
+    for i in range(2):
+        fd, cost = differences(shift(i))
+        assert np.all(np.abs(g["obs_center"][obs0, i] - fd) <= 1e-4 * np.abs(fd) + 1e-8 * cost + 1e-8), i
