@@ -767,8 +767,22 @@ __global__ void __launch_bounds__(kPostThreads) k_adj_post(AdjTrajArgs<T> a) {
 // reverse step k of the pair side.  Work decomposition of the forward pair
 // kernel: a CTA owns 32 (part, t) lanes of one scenario, warp w takes the
 // obstacles j = w, w+W, ...
+//
+// Bound by the latency of its loads: face by face, each value is used as soon as it
+// is read (8.4 of 14.5 cycles per issue on the long scoreboard).  STAGED: a warp copies the columns of its
+// next pair (y^{k+1}, y^k, ybar, zeta, xi and their adjoints, the obstacle's faces) to
+// shared memory while it works on this one, and the offset adjoints of eight faces
+// are summed over the lanes together instead of by five shuffles each.  Not STAGED
+// (two pairs of W warps exceed kAdjStageMax bytes): every value from global memory.
+// 256 trailer scenarios of 32 obstacles, FP32, 8 faces: 237 us a step, staged 154.
 // ============================================================================
-template <typename T, int D, int NR>
+constexpr size_t kAdjStageMax = 200 * 1024;
+// rows of 32 lanes of one staged pair
+__host__ __device__ inline int adj_pair_rows(int FR, int FO, int D) {
+    return 2 * (FR + FO + 1) + FO + 2 * (D + 1) + (FO * (D + 1) + 31) / 32;
+}
+
+template <typename T, int D, int NR, bool STAGED>
 __global__ void __launch_bounds__(256) k_adj_pair(AdjPairArgs<T> a) {
     constexpr int V = D + 1, NW = StatDims<D>::NW, PK = D + D * D;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -821,17 +835,68 @@ __global__ void __launch_bounds__(256) k_adj_pair(AdjPairArgs<T> a) {
 #pragma unroll
         for (int i = 0; i < D * D; ++i) Eb[i] = a.statsb[(long long)(NW + D + i) * a.Qtot + col];
 
+        // staged pair: rows of y^{k+1}, ybar, y^k (obstacle faces), (zeta, xi), their
+        // adjoints, then the obstacle's [C | d]
+        const int NY = FR + FO + 1, rY0 = 2 * NY, rZX = rY0 + FO, rZB = rZX + V, rOB = rZB + V;
+        const int rows = STAGED ? adj_pair_rows(FR, FO, D) : 0;
+        T *stage = red + (W * PK + warp * 2 * rows) * 32;
+        auto fetch = [&](int j, T *buf) {
+            const int gm = sm.obs0 + j, no = a.g.obs_nf[gm];
+            const long long p = sm.pair0 + (long long)j * Q + (valid ? q : Q - 1);
+            T *b = buf + lane;
+            for (int kk = 0; kk < nr; ++kk) {
+                cp_async_elem(b + kk * 32, a.y_k1 + p + (long long)kk * P);
+                cp_async_elem(b + (NY + kk) * 32, a.ybar_in + p + (long long)kk * P);
+            }
+            for (int m = 0; m < no; ++m) {
+                const long long at = p + (long long)(FR + m) * P;
+                cp_async_elem(b + (FR + m) * 32, a.y_k1 + at);
+                cp_async_elem(b + (NY + FR + m) * 32, a.ybar_in + at);
+                cp_async_elem(b + (rY0 + m) * 32, a.y_k + at);
+            }
+            cp_async_elem(b + (NY - 1) * 32, a.y_k1 + p + (long long)(NY - 1) * P);
+            cp_async_elem(b + (2 * NY - 1) * 32, a.ybar_in + p + (long long)(NY - 1) * P);
+#pragma unroll
+            for (int i = 0; i < V; ++i) cp_async_elem(b + (rZX + i) * 32, a.zx_k + p + (long long)i * P);
+            cp_async_elem(b + rZB * 32, a.zb + p);
+#pragma unroll
+            for (int i = 0; i < D; ++i) cp_async_elem(b + (rZB + 1 + i) * 32, a.xb + p + (long long)i * P);
+            for (int e = lane; e < no * D; e += 32) cp_async_elem(buf + rOB * 32 + e, a.g.obs_C + (long long)gm * FO * D + e);
+            for (int e = lane; e < no; e += 32) cp_async_elem(buf + rOB * 32 + FO * D + e, a.g.obs_d + (long long)gm * FO + e);
+            cp_async_commit();
+        };
+        int half = 0;
+        if constexpr (STAGED)
+            if (warp < sm.M) fetch(warp, stage);
+        // y rows: of the staged pair, or of global memory
+        const long long ys = STAGED ? 32 : P;
         for (int j = warp; j < sm.M; j += W) {
             const int gm = sm.obs0 + j;
-            const T *C = a.g.obs_C + (long long)gm * FO * D, *dd = a.g.obs_d + (long long)gm * FO;
             const int no = a.g.obs_nf[gm];
             const long long p = sm.pair0 + (long long)j * Q + (valid ? q : Q - 1);
-            const T *y1 = a.y_k1 + p, *y0 = a.y_k + p, *yi = a.ybar_in + p;
+            const T *C = a.g.obs_C + (long long)gm * FO * D, *dd = a.g.obs_d + (long long)gm * FO;
+            const T *y1 = a.y_k1 + p, *y0 = a.y_k + p + (long long)FR * P, *yi = a.ybar_in + p;
+            const T *zx = a.zx_k + p, *zbar = a.zb + p, *xbar = a.xb + p;
+            T *buf = stage + half * rows * 32;
+            if constexpr (STAGED) {
+                cp_async_wait_all();
+                __syncwarp();  // the obstacle's faces came by other lanes, which are also done with the other half
+                if (j + W < sm.M) fetch(j + W, stage + (half ^ 1) * rows * 32);
+                half ^= 1;
+                C = buf + rOB * 32;
+                dd = C + FO * D;
+                y1 = buf + lane;
+                yi = y1 + NY * 32;
+                y0 = y1 + rY0 * 32;
+                zx = y1 + rZX * 32;
+                zbar = y1 + rZB * 32;
+                xbar = zbar + 32;
+            }
             T *yo = a.ybar_out + p;
-            const T zeta = a.zx_k[p];
+            const T zeta = zx[0];
             T xi[D];
 #pragma unroll
-            for (int i = 0; i < D; ++i) xi[i] = a.zx_k[(long long)(1 + i) * P + p];
+            for (int i = 0; i < D; ++i) xi[i] = zx[(1 + i) * ys];
             // ---- pass 1: sums of y^{k+1}
             T lp[NR], a1[D], w1w[D], Sd = T(0);
 #pragma unroll
@@ -841,17 +906,17 @@ __global__ void __launch_bounds__(256) k_adj_pair(AdjPairArgs<T> a) {
             }
 #pragma unroll
             for (int kk = 0; kk < NR; ++kk) {
-                lp[kk] = kk < nr ? y1[(long long)kk * P] : T(0);
+                lp[kk] = kk < nr ? y1[kk * ys] : T(0);
 #pragma unroll
                 for (int i = 0; i < D; ++i) a1[i] += lp[kk] * ak[kk][i];
             }
             for (int m = 0; m < no; ++m) {
-                const T mp = y1[(long long)(FR + m) * P];
+                const T mp = y1[(FR + m) * ys];
 #pragma unroll
                 for (int i = 0; i < D; ++i) w1w[i] += mp * C[m * D + i];
                 Sd += mp * dd[m];
             }
-            const T gp1 = y1[(long long)(FR + FO) * P];
+            const T gp1 = y1[(FR + FO) * ys];
             // ---- statistics adjoint: W += w w^T, Wc += c w, E += w e^T
             const T cc = T(1) + Sd + gp1 + zeta;
             T e[D], w1b[D], eb[D], ccb = T(0);
@@ -886,9 +951,9 @@ __global__ void __launch_bounds__(256) k_adj_pair(AdjPairArgs<T> a) {
                 }
                 eb[jj] = acc;
             }
-            T zb = a.zb[p] + ccb, xb[D];
+            T zb = zbar[0] + ccb, xb[D];
 #pragma unroll
-            for (int i = 0; i < D; ++i) xb[i] = a.xb[(long long)i * P + p] + eb[i];
+            for (int i = 0; i < D; ++i) xb[i] = xbar[i * ys] + eb[i];
             // ---- the QP's dual point w* = K^T y^{k+1} + bq
             T wr = T(0);
 #pragma unroll
@@ -923,7 +988,7 @@ __global__ void __launch_bounds__(256) k_adj_pair(AdjPairArgs<T> a) {
             for (int i = 0; i < D; ++i) ba[i] = T(0);
 #pragma unroll
             for (int kk = 0; kk < NR; ++kk) {
-                T v = kk < nr ? yi[(long long)kk * P] : T(0);
+                T v = kk < nr ? yi[kk * ys] : T(0);
 #pragma unroll
                 for (int i = 0; i < D; ++i) v += ak[kk][i] * eb[i];
                 yol[kk] = v;
@@ -952,14 +1017,14 @@ __global__ void __launch_bounds__(256) k_adj_pair(AdjPairArgs<T> a) {
                 }
             }
             // slack gamma
-            const T yog = yi[(long long)(FR + FO) * P] + ccb;
+            const T yog = yi[(FR + FO) * ys] + ccb;
             if (gp1 > T(0)) {
                 H[0][0] += T(1);
                 rr[0] += yog;
             }
             // ---- pass 2: active obstacle faces
             for (int m = 0; m < no; ++m) {
-                const T mp = y1[(long long)(FR + m) * P];
+                const T mp = y1[(FR + m) * ys];
                 if (!(mp > T(0))) continue;
                 T c[D], cr = T(0), c2 = T(0), Km[V];
 #pragma unroll
@@ -977,7 +1042,7 @@ __global__ void __launch_bounds__(256) k_adj_pair(AdjPairArgs<T> a) {
                     for (int l = 0; l < D; ++l) acc += R[l * D + i] * c[l];
                     Km[1 + i] = acc;
                 }
-                T yom = yi[(long long)(FR + m) * P] + ccb * dm;
+                T yom = yi[(FR + m) * ys] + ccb * dm;
 #pragma unroll
                 for (int i = 0; i < D; ++i) yom += c[i] * w1b[i];
                 const T iDg = T(1) / (dpm * dpm + c2);
@@ -1018,7 +1083,7 @@ __global__ void __launch_bounds__(256) k_adj_pair(AdjPairArgs<T> a) {
                 wk[i] = T(0);
             }
             for (int m = 0; m < no; ++m) {
-                const T mp = y1[(long long)(FR + m) * P], mk = y0[(long long)(FR + m) * P];
+                const T mp = y1[(FR + m) * ys], mk = y0[m * ys];
                 T c[D], cr = T(0), c2 = T(0), cRw = T(0), cu = T(0), cRv = T(0), cw1b = T(0);
 #pragma unroll
                 for (int i = 0; i < D; ++i) {
@@ -1041,7 +1106,7 @@ __global__ void __launch_bounds__(256) k_adj_pair(AdjPairArgs<T> a) {
                 T dpb = mp * u[0];   // d/dd' of (K^T y).u at fixed y
                 T ybo = T(0);
                 if (mp > T(0)) {
-                    const T yom = yi[(long long)(FR + m) * P] + ccb * dm + cw1b;
+                    const T yom = yi[(FR + m) * ys] + ccb * dm + cw1b;
                     const T yh = yom + dpm * u[0] + cu;
                     const T iDg = T(1) / (rho_p * Dg), h = dpm * w0 + cRw;
                     ybo = yh;
@@ -1060,9 +1125,27 @@ __global__ void __launch_bounds__(256) k_adj_pair(AdjPairArgs<T> a) {
                 for (int i = 0; i < D; ++i) pb[i] -= dpb * c[i];
                 // offset adjoint: d' = d - c.rho, plus the statistics' c = 1 + d^T mu + ...
                 T gdv = valid ? dpb + ccb * mp : T(0);
+                if constexpr (STAGED) {
+                    buf[(FR + m) * 32 + lane] = gdv;  // over y^{k+1}'s, which is not read again
+                } else {
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) gdv += __shfl_xor_sync(0xffffffffu, gdv, o);
-                if (lane == 0) atomicAdd(a.gd + (long long)gm * FO + m, double(gdv));
+                    for (int o = 16; o > 0; o >>= 1) gdv += __shfl_xor_sync(0xffffffffu, gdv, o);
+                    if (lane == 0) atomicAdd(a.gd + (long long)gm * FO + m, double(gdv));
+                }
+            }
+            if constexpr (STAGED) {
+                // four lanes to a face, eight values to a lane; the start differs by face: no bank twice
+                __syncwarp();
+                for (int m0 = 0; m0 < no; m0 += 8) {
+                    const int m = m0 + (lane >> 2);
+                    T v = T(0);
+                    if (m < no)
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) v += buf[(FR + m) * 32 + (lane & 3) * 8 + ((i + (lane >> 2)) & 7)];
+                    v += __shfl_xor_sync(0xffffffffu, v, 1);
+                    v += __shfl_xor_sync(0xffffffffu, v, 2);
+                    if (m < no && (lane & 3) == 0) atomicAdd(a.gd + (long long)gm * FO + m, double(v));
+                }
             }
             // R adjoint: -sum_act yh c w1*^T / (rho Dg) + w+ u1^T + [head] w^k xi_bar^T
 #pragma unroll
@@ -1267,8 +1350,16 @@ cudaError_t launch_adj_traj(const AdjTrajArgs<T> &a, int n_scen, int *lq_ok, con
 
 template <typename T, int D, int NR>
 cudaError_t launch_adj_pair_t(const AdjPairArgs<T> &a, int n_tiles, int W, cudaStream_t st) {
-    const size_t sm = (size_t)W * (D + D * D) * 32 * sizeof(T);
-    k_adj_pair<T, D, NR><<<n_tiles, dim3(32, W), sm, st>>>(a);
+    const size_t red = (size_t)W * (D + D * D) * 32 * sizeof(T);
+    const size_t staged = red + (size_t)W * 2 * adj_pair_rows(a.g.FR, a.g.FO, D) * 32 * sizeof(T);
+    if (staged <= kAdjStageMax) {
+        const cudaError_t e = cudaFuncSetAttribute(k_adj_pair<T, D, NR, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   int(kAdjStageMax));
+        if (e != cudaSuccess) return e;
+        k_adj_pair<T, D, NR, true><<<n_tiles, dim3(32, W), staged, st>>>(a);
+    } else {
+        k_adj_pair<T, D, NR, false><<<n_tiles, dim3(32, W), red, st>>>(a);
+    }
     return cudaGetLastError();
 }
 

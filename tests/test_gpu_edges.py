@@ -112,3 +112,63 @@ def test_cold_start_on_the_device(B, dtype):
     for sc in (_mixed(dtype), synth.config3(n_scen=5), synth.config4(n_scen=2, n_obs=8, N=5), synth.config_max()):
         ds = B.DeviceScene(B.Context(0), sc, dtype)
         assert torch.equal(ds.cold_y(), ds.to_device_pairs(sc.cold_y()))
+
+
+def _faces_scene(dim, faces, n_obs, N):
+    """One scenario whose obstacles all have `faces` faces."""
+    rng = np.random.default_rng([31, dim, faces, n_obs])
+    if dim == 2:
+        model = synth.trailer_model()
+        return synth._assemble(model, [synth._trailer_scen(rng, model, N, n_obs, faces, faces, 2.0 * N, 20.0, 2)], "faces")
+    model = synth.quad_model()
+    obs = []
+    for _ in range(n_obs):
+        C, off = synth.random_polyhedron(rng, faces, 0.3, 0.6)
+        obs.append((C, off, np.array([rng.uniform(1.0, 3.0), rng.uniform(-1.5, 1.5), rng.uniform(1.5, 3.5)])))
+    ref = np.zeros((N + 1, model.ns))
+    ref[:, 2] = 2.5
+    ref[:, 0] = 4.0 * np.arange(N + 1) / N
+    ref[:, 3] = 4.0 / (N * model.dt)
+    return synth._assemble(model, [synth._Scen(obs, synth._quad_parts(), N, ref, np.zeros((N, model.nu)))], "faces")
+
+
+# faces: fewer than the eight summed together, eight, a second group, three; the last
+# one is too large to be staged in FP64; obstacles: one warp, fewer and more than warps
+FACES = [(2, 3, 1, 5), (2, 8, 5, 20), (2, 9, 9, 17), (2, 24, 20, 8), (3, 7, 3, 7), (3, 24, 9, 5)]
+
+
+def _face_differences(ora, sc, K, kw, pairs, h=1e-4):
+    """Central differences of the oracle's cost by obstacle offsets (step 1e-4: see the
+    trajectory split's gradient test)."""
+    import dataclasses
+    out = []
+    for j, m in pairs:
+        costs = []
+        for e in (h, -h):
+            d = sc.obs_d.copy()
+            d[j, m] += e
+            costs.append(ora.admm_batch(dataclasses.replace(sc, obs_d=d), max_iter=K, **kw)["cost"].sum())
+        out.append((j, m, (costs[0] - costs[1]) / (2 * h), abs(costs[0])))
+    return out
+
+
+GRAD_KW = dict(sigma=300.0, eps_pri=0.0, eps_dual=0.0, prox=0.1, rho_box=100.0, damp=100.0)
+
+
+@pytest.mark.parametrize("dim,faces,n_obs,N", FACES)
+def test_pair_adjoint_face_counts(B, ora, dim, faces, n_obs, N):
+    """Offset gradients of staged and unstaged pairs against central differences of the
+    oracle (FP64; the tolerance of the trajectory split's gradient test)."""
+    sc, K = _faces_scene(dim, faces, n_obs, N), 3
+    ds = B.DeviceScene(B.Context(0), sc, torch.float64)
+    pb = B.Problem(ds)
+    tape = B.new_tape(ds, K)
+    rep = B.admm_solve(ds, pb.s_ref, pb.s, pb.u, pb.y, pb.zeta, pb.xi, tape=tape, max_iter=K, **GRAD_KW)
+    g = B.admm_backward(ds, pb.s_ref, tape, rep["iters"], torch.ones(1, dtype=torch.float64, device=ds.device),
+                        max_iter=K, **{k: GRAD_KW[k] for k in ("sigma", "prox", "rho_box", "damp")})
+    got = g["obs_offset"].cpu().numpy()
+    # the corners of the table and its five largest entries
+    pairs = {(j, m) for j in (0, n_obs - 1) for m in (0, faces // 2, faces - 1)}
+    pairs |= {(int(i) // got.shape[1], int(i) % got.shape[1]) for i in np.argsort(-np.abs(got).ravel())[:5]}
+    for j, m, fd, cost in _face_differences(ora, sc, K, GRAD_KW, sorted(pairs)):
+        assert abs(got[j, m] - fd) <= 1e-4 * abs(fd) + 1e-8 * cost + 1e-8, (j, m, got[j, m], fd)
