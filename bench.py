@@ -374,9 +374,9 @@ def gpu_arm(args):
         # measured DRAM bytes per pair, scaled to the pairs an average launch processed
         traffic = float(kv["dram_bytes_per_pair"]) * tot[7] / tot[6]
     # per step: reset, 2 box inits, poses, gather, scale-detect poses + LP,
-    # certificate margin = 8, and per iteration launch: pair kernel,
-    # trajectory kernel, counter advance
-    launches = int(8 * args.steps * world + 3 * tot[6])
+    # certificate margin = 8, and per iteration launch: pair kernel and the
+    # trajectory step's three
+    launches = int(8 * args.steps * world + 4 * tot[6])
     n_sm = torch.cuda.get_device_properties(local).multi_processor_count
     sm_mhz = clk["sm_mhz"] if clk else 2070.0
 
@@ -441,7 +441,7 @@ def traj_roofline(scene, stages, traj_ms, fp64):
     f_stage = ric_flops_per_stage(scene.model.ns, scene.model.nu)
     ach = f_stage * stages / (traj_ms / 1e3) / 1e9
     return {"bound": "fp64", "achieved": ach, "peak": fp64, "unit": "GFLOP/s", "frac": ach / fp64 if fp64 > 0 else None,
-            "kernel": "k_riccati (FP64 backward Riccati recursion + forward sweep; the FP32 stage assembly not counted)",
+            "kernel": "k_traj_lq (FP64 backward Riccati recursion + forward sweep; launch time includes the stage assembly and update)",
             "flops_per_stage": f_stage, "stages": stages,
             "peak_source": "measured on this GPU (oca_fp64_peak: FP64 FMA microbenchmark)"}
 
