@@ -774,7 +774,7 @@ __global__ void __launch_bounds__(kPostThreads) k_adj_post(AdjTrajArgs<T> a) {
 // shared memory while it works on this one, and the offset adjoints of eight faces
 // are summed over the lanes together instead of by five shuffles each.  Not STAGED
 // (two pairs of W warps exceed kAdjStageMax bytes): every value from global memory.
-// 256 trailer scenarios of 32 obstacles, FP32, 8 faces: 237 us a step, staged 160.
+// 256 trailer scenarios of 32 obstacles, FP32, 3-12 faces: 237 us a step, staged 160.
 // ============================================================================
 constexpr size_t kAdjStageMax = 200 * 1024;
 // rows of 32 lanes of one staged pair
