@@ -499,17 +499,16 @@ __global__ void __launch_bounds__(kTrajBlock) k_traj_stage(RicArgs<T> a) {
     constexpr int NS = MDims<KIND>::NS;
     using Mp = RicMap<KIND>;
     const int s = blockIdx.x, lane = threadIdx.x, NT = blockDim.x;
-    if (a.scen_status[s] != kActive) return;
-    const int j = *a.iter;
-    if (j > a.max_iter) return;
     const ScenMeta sm = a.meta[s];
-    __shared__ int s_retired;
+    // one warp reads and writes the scenario's status; the others take its verdict
+    __shared__ int s_skip;
     if (lane < 32) {
-        const bool r = stop_rule<T, KIND>(a, sm, s, j);
-        if (lane == 0) s_retired = r;
+        const int j = *a.iter;
+        const bool skip = a.scen_status[s] != kActive || j > a.max_iter || stop_rule<T, KIND>(a, sm, s, j);
+        if (lane == 0) s_skip = skip;
     }
     __syncthreads();
-    if (s_retired) return;
+    if (s_skip) return;
     F *scr = reinterpret_cast<F *>(a.scratch) + a.scratch0[s];
     StageParams<T> sp;
     StageSrc<T> src;
