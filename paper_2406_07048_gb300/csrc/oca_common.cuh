@@ -12,6 +12,17 @@ constexpr int kMaxFO = OCA_MAX_OBS_FACES;
 constexpr int kMaxFR = OCA_MAX_PART_FACES;
 constexpr int kActive = OCA_SCEN_ACTIVE;
 
+// Dynamic shared memory beyond the 48 KB that any launch may use has to be allowed, and the
+// allowance belongs to the kernel: it is always the block's whole 227 KB (for kernels
+// without static shared memory), never one call's need, which another host thread's smaller
+// call could lower between this thread's allowance and its launch.
+constexpr int kMaxSmem = 227 * 1024;
+template <class Kernel>
+cudaError_t allow_smem(Kernel *kernel, size_t bytes) {
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(reinterpret_cast<const void *>(kernel), cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+}
+
 // Per-scenario metadata on the device.
 struct ScenMeta {
     int N;       // horizon N_s (constraint steps t = 1..N)

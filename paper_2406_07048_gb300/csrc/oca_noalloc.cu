@@ -146,11 +146,7 @@ oca_status run(const oca_scene_desc *d, const oca_model *m, void *scratch, const
     const int W = sc.M >= 32 ? 4 : (sc.M >= 8 ? 2 : 1);
     const unsigned tiles = (unsigned)((sc.Q + 31) / 32);
     const size_t sm = sizeof(T) * kLpRec * 32 * (size_t)W * (g.FR + g.FO);
-    if (sm > 48 * 1024 &&
-        cudaFuncSetAttribute(d->dim == 2 ? reinterpret_cast<const void *>(k_scale_one<T, 2>)
-                                         : reinterpret_cast<const void *>(k_scale_one<T, 3>),
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
-        return OCA_ERR_CUDA;
+    if (allow_smem(d->dim == 2 ? k_scale_one<T, 2> : k_scale_one<T, 3>, sm) != cudaSuccess) return OCA_ERR_CUDA;
     if (d->dim == 2)
         k_scale_one<T, 2><<<tiles, dim3(32, W), sm, st>>>(sc, g, pose, static_cast<T *>(alpha), static_cast<T *>(lambda),
                                                         static_cast<T *>(mu), verdict, status);

@@ -829,10 +829,8 @@ template <typename T, int D, int MODE, int SOLVER, int NR>
 cudaError_t launch_pair_t(const PairArgs<T> &a, int n_tiles, int W, cudaStream_t st) {
     if (n_tiles <= 0) return cudaSuccess;
     const size_t sm = pair_smem<T, D>(W, MODE, SOLVER, a.g.FR, a.g.FO);
-    if (sm > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_pair<T, D, MODE, SOLVER, NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(k_pair<T, D, MODE, SOLVER, NR>, sm);
+    if (e != cudaSuccess) return e;
     k_pair<T, D, MODE, SOLVER, NR><<<n_tiles, dim3(32, W), sm, st>>>(a);
     return cudaGetLastError();
 }
@@ -859,11 +857,8 @@ cudaError_t launch_scale(const ScaleArgs<T> &a, int dim, int n_tiles, int W, cud
     // warps then sweep the same obstacles
     size_t sm = scale_smem_bytes<T>(W, a.g.FR, a.g.FO);
     while (W > 1 && sm > 200 * 1024) sm = scale_smem_bytes<T>(--W, a.g.FR, a.g.FO);
-    const void *fn = dim == 2 ? reinterpret_cast<const void *>(k_scale<T, 2>) : reinterpret_cast<const void *>(k_scale<T, 3>);
-    if (sm > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(dim == 2 ? k_scale<T, 2> : k_scale<T, 3>, sm);
+    if (e != cudaSuccess) return e;
     if (dim == 2) k_scale<T, 2><<<n_tiles, dim3(32, W), sm, st>>>(a);
     else k_scale<T, 3><<<n_tiles, dim3(32, W), sm, st>>>(a);
     return cudaGetLastError();

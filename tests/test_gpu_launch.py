@@ -1,0 +1,96 @@
+"""Launch configuration of the tile kernels, read from captured launches (a stream capture
+records the kernel nodes; nothing of it is run)."""
+import ctypes as C
+
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2406_07048_gb300 import synth
+from tests.test_gpu_edges import _faces_scene, _mixed
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2406_07048_gb300 import _build, binding
+    _build.build()
+    return binding
+
+
+class _KernelNode(C.Structure):
+    _fields_ = [("func", C.c_void_p), ("grid", C.c_uint * 3), ("block", C.c_uint * 3), ("shared", C.c_uint),
+                ("params", C.c_void_p), ("extra", C.c_void_p), ("kern", C.c_void_p), ("ctx", C.c_void_p)]
+
+
+def _launches(call):
+    """The kernel launches of call(stream=...): (block, dynamic shared bytes, a function that
+    reads the kernel's limit of dynamic shared memory)."""
+    cu = C.CDLL("libcuda.so.1")
+    ok = lambda r: r == 0 or pytest.fail(f"driver call: {r}")
+    call(stream=None)  # allocations, and what is looked up once
+    torch.cuda.synchronize()
+    st, graph, n = torch.cuda.Stream(), C.c_void_p(), C.c_size_t(0)
+    ok(cu.cuStreamBeginCapture_v2(C.c_void_p(st.cuda_stream), 2))
+    try:
+        out = call(stream=st)
+    finally:
+        r = cu.cuStreamEndCapture(C.c_void_p(st.cuda_stream), C.byref(graph))
+    ok(r)
+    ok(cu.cuGraphGetNodes(graph, None, C.byref(n)))
+    nodes = (C.c_void_p * n.value)()
+    ok(cu.cuGraphGetNodes(graph, nodes, C.byref(n)))
+    found = []
+    for node in nodes:
+        kind = C.c_int()
+        ok(cu.cuGraphNodeGetType(C.c_void_p(node), C.byref(kind)))
+        if kind.value != 0:
+            continue
+        p = _KernelNode()
+        ok(cu.cuGraphKernelNodeGetParams_v2(C.c_void_p(node), C.byref(p)))
+        func = C.c_void_p(p.func)
+        if not func:
+            ok(cu.cuKernelGetFunction(C.byref(func), C.c_void_p(p.kern)))
+
+        def limit(func=func):
+            v = C.c_int()
+            ok(cu.cuFuncGetAttribute(C.byref(v), 8, func))
+            return v.value
+
+        found.append((tuple(p.block), p.shared, limit))
+    ok(cu.cuGraphDestroy(graph))
+    del out
+    return found
+
+
+def _states(ds):
+    return ds.tensor(ds.scene.s_init)
+
+
+@pytest.mark.parametrize("entry", ["scale", "noalloc", "pair"])
+def test_a_smaller_call_leaves_the_shared_memory_limit(B, entry):
+    """The limit of dynamic shared memory belongs to the kernel, not to the call: a call with
+    less of it must not lower the limit below that of a call that another thread is about to
+    launch (both calls need more than the 48 KB that need no limit)."""
+    ctx = B.Context(0)
+    scene = lambda sc, dtype: B.DeviceScene(ctx, sc, dtype)
+    if entry == "scale":
+        big, small = scene(_mixed(torch.float32), torch.float32), scene(_faces_scene(2, 8, 16, 5), torch.float32)
+        run = lambda ds: lambda stream: B.scale_detect(ds, _states(ds), stream=stream)
+    elif entry == "noalloc":
+        big, small = (scene(_faces_scene(2, f, 33, 5), torch.float64) for f in (24, 12))
+        run = lambda ds: lambda stream: B.scale_detect_noalloc(ds, _states(ds), stream=stream)
+    else:
+        big, small = (scene(_faces_scene(2, f, 16, 5), torch.float32) for f in (24, 9))
+        big.warps = small.warps = 8
+
+        def run(ds):
+            pb = B.Problem(ds)
+            return lambda stream: B.pair_qp(ds, pb.s, pb.zeta, pb.xi, pb.y, prox=1.0, stream=stream)
+    _, need, limit = max(_launches(run(big)), key=lambda f: f[1])
+    after = max(shared for _, shared, _ in _launches(run(small)))
+    assert 48 * 1024 < after < need
+    assert limit() >= need
