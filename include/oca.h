@@ -145,8 +145,7 @@ oca_status oca_scene_info_get(const oca_scene *scene, oca_scene_info *info);
 /* Work shape of the pair kernels: warps per 32-lane tile (1..16); each warp
  * sweeps every W-th obstacle of the tile's scenario.  oca_scene_create picks
  * it from the number of tiles (few tiles: up to one warp per obstacle, many:
- * two), and another for the LP and margin kernels; a count set here holds for
- * all of them.  DeviceScene.autotune_warps in the Python binding times the fused pair
+ * two).  DeviceScene.autotune_warps in the Python binding times the fused pair
  * kernel of short solves for each candidate and sets the fastest.
  * Errors: OCA_ERR_INVALID_ARGUMENT (warps outside 1..16), OCA_ERR_CAPACITY
  * (more warps per tile than the pair kernels are compiled for -- 16 for
@@ -158,6 +157,14 @@ oca_status oca_scene_info_get(const oca_scene *scene, oca_scene_info *info);
  * in 3-D, nstat = 9 in 2-D and 18 in 3-D). */
 oca_status oca_scene_set_warps(oca_scene *scene, int warps);
 int oca_scene_get_warps(const oca_scene *scene); /* -1 if scene == NULL */
+
+/* The same of the scale LP and margin kernels (oca_scale_detect_batch,
+ * oca_cert_margin_batch), which have a count of their own: setting one leaves
+ * the other.  A count whose staged LP columns do not fit the device's shared
+ * memory is lowered for that launch.
+ * Errors: OCA_ERR_INVALID_ARGUMENT (warps outside 1..16). */
+oca_status oca_scene_set_lp_warps(oca_scene *scene, int warps);
+int oca_scene_get_lp_warps(const oca_scene *scene); /* -1 if scene == NULL */
 
 /* ------------------------------------------------------------------------ */
 /* Model and ADMM parameters                                                */

@@ -73,8 +73,8 @@ class Report(C.Structure):
 
 
 EXPORTED = ["oca_create", "oca_destroy", "oca_status_string", "oca_scene_create", "oca_scene_destroy",
-            "oca_scene_info_get", "oca_scene_set_warps", "oca_scene_get_warps", "oca_scale_detect_batch",
-            "oca_pair_qp_batch", "oca_admm_solve", "oca_profile_enable", "oca_profile_read",
+            "oca_scene_info_get", "oca_scene_set_warps", "oca_scene_get_warps", "oca_scene_set_lp_warps",
+            "oca_scene_get_lp_warps", "oca_scale_detect_batch", "oca_pair_qp_batch", "oca_admm_solve", "oca_profile_enable", "oca_profile_read",
             "oca_scale_detect_noalloc", "oca_admm_tape_bytes", "oca_admm_solve_taped", "oca_admm_backward",
             "oca_mpc_run", "oca_pair_qp_lemke_batch", "oca_admm_fixed_point_tape_bytes", "oca_fp64_peak",
             "oca_cert_margin_batch", "oca_lq_workspace_bytes", "oca_lq_solve"]
@@ -104,6 +104,10 @@ def lib():
         L.oca_scene_set_warps.restype = I
         L.oca_scene_get_warps.argtypes = [P]
         L.oca_scene_get_warps.restype = I
+        L.oca_scene_set_lp_warps.argtypes = [P, I]
+        L.oca_scene_set_lp_warps.restype = I
+        L.oca_scene_get_lp_warps.argtypes = [P]
+        L.oca_scene_get_lp_warps.restype = I
         L.oca_scale_detect_batch.argtypes = [P, P, C.POINTER(ModelC), P, P, P, P, P, P, P, P]
         L.oca_scale_detect_batch.restype = I
         L.oca_cert_margin_batch.argtypes = [P, P, C.POINTER(ModelC), P, P, P, P, P]
@@ -262,7 +266,7 @@ class DeviceScene:
             setattr(d, name, getattr(self.desc, name))
         d.obs_d = new.obs_d.data_ptr()
         new._create(d, self.device)
-        new.warps = self.warps
+        new.warps, new.lp_warps = self.warps, self.lp_warps
         return new
 
     def autotune_warps(self, problem: "Problem", params: Optional[dict] = None,
@@ -309,6 +313,15 @@ class DeviceScene:
     @warps.setter
     def warps(self, w: int):
         _check(lib().oca_scene_set_warps(self.h, int(w)), "oca_scene_set_warps")
+
+    @property
+    def lp_warps(self) -> int:
+        """Warps per tile of the scale LP and margin kernels."""
+        return int(lib().oca_scene_get_lp_warps(self.h))
+
+    @lp_warps.setter
+    def lp_warps(self, w: int):
+        _check(lib().oca_scene_set_lp_warps(self.h, int(w)), "oca_scene_set_lp_warps")
 
     def close(self):
         if getattr(self, "h", None):

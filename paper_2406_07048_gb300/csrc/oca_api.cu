@@ -1209,11 +1209,19 @@ oca_status oca_scene_info_get(const oca_scene *sc, oca_scene_info *info) {
 oca_status oca_scene_set_warps(oca_scene *sc, int warps) {
     if (!sc || warps < 1 || warps > 16) return OCA_ERR_INVALID_ARGUMENT;
     if (!warps_fit(sc, warps)) return OCA_ERR_CAPACITY;
-    sc->W = sc->W_lp = warps;
+    sc->W = warps;
     return OCA_OK;
 }
 
 int oca_scene_get_warps(const oca_scene *sc) { return sc ? sc->W : -1; }
+
+oca_status oca_scene_set_lp_warps(oca_scene *sc, int warps) {
+    if (!sc || warps < 1 || warps > 16) return OCA_ERR_INVALID_ARGUMENT;
+    sc->W_lp = warps;
+    return OCA_OK;
+}
+
+int oca_scene_get_lp_warps(const oca_scene *sc) { return sc ? sc->W_lp : -1; }
 
 oca_status oca_scale_detect_batch(oca_ctx *ctx, const oca_scene *scene, const oca_model *model, const void *states,
                                   void *alpha, void *lambda, void *mu, double *margin, int32_t *verdict,

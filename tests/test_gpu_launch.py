@@ -94,3 +94,34 @@ def test_a_smaller_call_leaves_the_shared_memory_limit(B, entry):
     after = max(shared for _, shared, _ in _launches(run(small)))
     assert 48 * 1024 < after < need
     assert limit() >= need
+
+
+def test_warps_of_the_pair_and_of_the_lp_kernels(B):
+    """The pair kernels' count of warps, set or tuned, leaves the LP and margin kernels'
+    count, also on a scene derived with other offsets; theirs changes no result."""
+    ds = B.DeviceScene(B.Context(0), synth.config3(n_scen=64), torch.float32)
+    pb = B.Problem(ds)
+
+    def lp_warps(ds):
+        out = B.scale_detect(ds, pb.s)
+        shapes = _launches(lambda stream: B.scale_detect(ds, pb.s, stream=stream))
+        shapes += _launches(lambda stream: B.cert_margin(ds, pb.s, out["lam"], out["mu"], stream=stream))
+        return sorted(block[1] for block, _, _ in shapes if block[0] == 32)
+
+    own = lp_warps(ds)
+    assert len(own) == 2 and own[0] == own[1] > 2
+    ds.warps = 2
+    assert lp_warps(ds) == own
+    assert lp_warps(ds.with_offsets(ds.obs_d)) == own
+    ds.autotune_warps(pb, candidates=(1, 3), iters=1)
+    assert lp_warps(ds) == own
+    ref = B.scale_detect(ds, pb.s)
+    for w in (1, 5):
+        ds.lp_warps = w
+        assert lp_warps(ds) == [w, w] == lp_warps(ds.with_offsets(ds.obs_d))
+        got = B.scale_detect(ds, pb.s)
+        assert all(torch.equal(got[k], ref[k]) for k in ref)
+        assert torch.equal(B.cert_margin(ds, pb.s, got["lam"], got["mu"]), B.cert_margin(ds, pb.s, ref["lam"], ref["mu"]))
+    with pytest.raises(B.OcaError) as e:
+        ds.lp_warps = 17
+    assert e.value.code == 1
