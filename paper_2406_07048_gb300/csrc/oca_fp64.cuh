@@ -1,0 +1,26 @@
+// FP64 operations for the chains of the LQ solves, where an FP64 instruction holds a
+// scheduler for 64 cycles whatever its lanes do.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace oca {
+
+// 1 / x by one step of the third-order hyperpower iteration, y <- y + y (e + e^2) with
+// e = 1 - x y (M. Altman, Pacific J. Math. 10, 1960; its second-order form is Schulz's),
+// from the hardware's approximation.  That one keeps the upper 32 bits of its operand and
+// of its result, so |e| < 2^-19 and what the step leaves, e^3, is below 2^-57 of 1 / x:
+// with the rounding of the last multiply-add at most 0.57 units in the last place.  Three
+// multiply-adds; the approximation flushes subnormal numbers, so where x or 1 / x is near
+// them (|x| < 2^-1021 or |x| >= 2^1021, and not finite) the quotient is formed by division.
+__device__ __forceinline__ double recip(double x) {
+    const unsigned ex = (unsigned)__double2hiint(x) >> 20 & 0x7ffu;
+    if (ex - 2u > 2041u) return 1.0 / x;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ float recip(float x) { return 1.0f / x; }
+
+}  // namespace oca

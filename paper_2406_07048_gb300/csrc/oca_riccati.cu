@@ -20,6 +20,7 @@
 #include <type_traits>
 
 #include "oca_common.cuh"
+#include "oca_fp64.cuh"
 #include "oca_kernels.h"
 #include "oca_ric.cuh"
 #include "oca_ricprog.cuh"
@@ -185,16 +186,6 @@ __device__ constexpr auto kRicTab = RicBuild<KIND>::template table<PHASE, L>();
 template <int KIND>
 __device__ constexpr auto kRicOut = RicBuild<KIND>::out_map();
 
-// 1 / x by one step of the third-order Newton-Schulz iteration
-// y <- y + y (e + e^2), e = 1 - x y, from the hardware's approximation: the error
-// e (about 2^-20) becomes e^3 < 2^-53 with three multiply-adds
-__device__ __forceinline__ double lq_rcp(double x) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
-__device__ __forceinline__ float lq_rcp(float x) { return 1.0f / x; }
 // x > 0 and x finite on the integer pipe (an FP64 compare costs as much as a multiply-add)
 __device__ __forceinline__ bool lq_positive(double x) {
     const long long b = __double_as_longlong(x);
@@ -651,7 +642,7 @@ __global__ void __launch_bounds__(32 * kLqWarps) k_traj_lq(LqArgs2<F> a) {
             const F det = fma(u00, u11, -(u01 * u01));
             const bool pd = lq_positive(u00) && lq_positive(det);
             ok = ok && pd;
-            const F id = pd ? -lq_rcp(det) : F(0);
+            const F id = pd ? -recip(det) : F(0);
 #pragma unroll
             for (int r = 0; r < PK; ++r) {
                 const int e = li + L * r;
@@ -793,7 +784,7 @@ __global__ void __launch_bounds__(128) k_traj_lq4(LqArgs2<F> a) {
                 for (int i = 0; i < NU; ++i) col[i] = __shfl_sync(0xffffffffu, v[i], c);
                 const bool pd = lq_positive(col[c]);
                 ok = ok && pd;
-                v[c] *= pd ? lq_rcp(col[c]) : F(1);
+                v[c] *= pd ? recip(col[c]) : F(1);
 #pragma unroll
                 for (int i = 0; i < NU; ++i)
                     if (i != c) v[i] = fma(-col[i], v[c], v[i]);

@@ -36,6 +36,7 @@
 #include <utility>
 
 #include "oca_common.cuh"
+#include "oca_fp64.cuh"
 #include "oca_kernels.h"
 
 namespace oca {
@@ -63,14 +64,6 @@ __host__ __device__ inline int lq_es(int n) { return 3 * n * n + 2 * n; }
 // entry to a thread, small systems are solved with one column per lane, compares
 // run on the integer pipe and a reciprocal is three multiply-adds.
 
-// 1 / x by one third-order Newton-Schulz step y + y (e + e^2), e = 1 - x y, from the
-// hardware's approximation (e about 2^-20, so e^3 < 2^-53)
-__device__ __forceinline__ double fast_rcp(double x) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
 // order of |x| as an integer (NaN above infinity)
 __device__ __forceinline__ unsigned long long abs_bits(double x) {
     return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
@@ -119,7 +112,7 @@ __device__ __forceinline__ bool gj_columns(double (&v)[kLqMaxU], int m, int lane
         double col[kLqMaxU];
 #pragma unroll
         for (int i = 0; i < kLqMaxU; ++i) col[i] = i < m ? __shfl_sync(0xffffffffu, v[i], c) : 0.0;
-        v[c] *= fast_rcp(fine ? col[c] : 1.0);
+        v[c] *= recip(fine ? col[c] : 1.0);
 #pragma unroll
         for (int i = 0; i < kLqMaxU; ++i)
             if (i != c && i < m) v[i] = fma(-col[i], v[c], v[i]);
@@ -246,7 +239,7 @@ __global__ void __launch_bounds__(kLqThreads) k_lq_compose(LqArgs a, const doubl
         const double pv = S[px * W + pc];
         const bool fine = abs_bits(pv) > 0x01a56e1fc2f8f359ull && abs_bits(pv) < 0x7ff0000000000000ull;  // > 1e-300, finite
         bad = bad || !fine;
-        const double ip = fast_rcp(fine ? pv : 1.0);
+        const double ip = recip(fine ? pv : 1.0);
         // a lane per column (the columns past 32 in a second pass while they are
         // active), the rows dealt over the warps: the scaled pivot row is formed once
         // per column and warp

@@ -1,0 +1,83 @@
+"""The FP64 operations that the LQ solves form without a division or a compare
+(oca_fp64.cuh), against IEEE arithmetic over the whole range of their operands, and the
+entry points at operands near the ends of that range."""
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture(scope="module")
+def B():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2406_07048_gb300 import _build, binding
+    _build.build()
+    return binding
+
+
+@pytest.fixture(scope="module")
+def ops(B, tmp_path_factory):
+    from paper_2406_07048_gb300 import _build
+    so = str(tmp_path_factory.mktemp("fp64") / "fp64.so")
+    r = subprocess.run([_build.nvcc()] + _build.ARCH + _build.FLAGS + ["-shared", "-o", so,
+                       os.path.join(ROOT, "tests", "gpu", "fp64.cu")], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+    return C.CDLL(so)
+
+
+def _apply(fn, x, out):
+    xt = torch.as_tensor(x, device="cuda")
+    yt = torch.zeros(len(x), dtype=out, device="cuda")
+    assert fn(C.c_void_p(xt.data_ptr()), C.c_void_p(yt.data_ptr()), C.c_int(len(x)),
+              C.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+    return yt.cpu().numpy()
+
+
+def _operands():
+    """Every exponent, subnormal ones among them, with random mantissas, the smallest and
+    the largest; both signs."""
+    rng = np.random.default_rng(11)
+    bits = [np.uint64(e) << np.uint64(52) | m for e in range(2047)
+            for m in (np.uint64(0), np.uint64(1), np.uint64(2**52 - 1), *rng.integers(0, 2**52, 40, dtype=np.uint64))]
+    x = np.array(bits, dtype=np.uint64).view(np.float64)
+    return np.concatenate([x, -x])
+
+
+def test_recip_over_the_range(ops):
+    """At most 0.57 units in the last place from 1 / x, whose own rounding moves the
+    quotient by half a unit: not more than one number away from the correctly rounded one;
+    the same number where 1 / x is formed by division."""
+    x = _operands()
+    with np.errstate(divide="ignore", over="ignore"):
+        want = 1.0 / x
+    got = _apply(ops.run_recip, x, torch.float64)
+    sub = (np.abs(x) < 2.0**-1021) | (np.abs(x) >= 2.0**1021)
+    assert (got[sub].view(np.int64) == want[sub].view(np.int64)).all()
+    away = np.abs(got[~sub].view(np.int64) - want[~sub].view(np.int64))
+    print(f"[recip] {np.mean(away != 0):.3g} of the quotients are not the rounded one")
+    assert away.max() <= 1
+    got = _apply(ops.run_recip, np.array([np.inf, -np.inf, np.nan]), torch.float64)
+    assert got[0] == 0.0 and got[1] == 0.0 and np.isnan(got[2])
+
+
+@pytest.mark.parametrize("method", [0, 1])
+def test_lq_with_a_huge_control_cost(B, method):
+    """R = 1.5e308, r = 1e308 and controls that reach no state: u = -r / R (the reciprocal of
+    R is a subnormal number of 51 bits: 1e-14)."""
+    N, ns, nu = 3, 2, 2
+    z = lambda *shape: torch.zeros(1, *shape, dtype=torch.float64, device="cuda")
+    eye = lambda n, k: torch.eye(n, dtype=torch.float64, device="cuda").repeat(1, k, 1, 1)
+    out = B.lq_solve(B.Context(0), eye(ns, N), z(N, ns, nu), z(N, ns), eye(ns, N + 1), z(N + 1, ns),
+                     1.5e308 * eye(nu, N), z(N, nu) + 1e308, z(ns) + 1.0, method=method)
+    torch.cuda.synchronize()
+    assert int(out["status"][0]) == 0
+    assert (out["u"] + 1e308 / 1.5e308).abs().max().item() <= 1e-14
