@@ -13,13 +13,15 @@ namespace oca {
 // with the rounding of the last multiply-add at most 0.57 units in the last place.  Three
 // multiply-adds; the approximation flushes subnormal numbers, so where x or 1 / x is near
 // them (|x| < 2^-1021 or |x| >= 2^1021, and not finite) the quotient is formed by division.
+// The test comes last, off the chain: 256 problems of 64 stages 386 -> 382 us (379 without).
 __device__ __forceinline__ double recip(double x) {
-    const unsigned ex = (unsigned)__double2hiint(x) >> 20 & 0x7ffu;
-    if (ex - 2u > 2041u) return 1.0 / x;
     double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    asm volatile("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
+    y = fma(y, fma(e, e, e), y);
+    const unsigned ex = (unsigned)__double2hiint(x) >> 20 & 0x7ffu;
+    if (__builtin_expect(ex - 2u > 2041u, 0)) y = 1.0 / x;
+    return y;
 }
 __device__ __forceinline__ float recip(float x) { return 1.0f / x; }
 
