@@ -637,19 +637,20 @@ __global__ void __launch_bounds__(32 * kLqWarps) k_traj_lq(LqArgs2<F> a) {
         __syncwarp();
         if (act) {
             // K = -Quu^-1 [Qus | qu] by the 2 x 2 adjugate; Quu not positive definite: K = 0, the
-            // scenario fails
+            // scenario fails.  The inverse is formed before its product: u11 [Qus | qu] may
+            // pass the largest number where det does not.
             const F u00 = sm[Mp::U0], u01 = sm[Mp::U0 + 1], u11 = sm[Mp::U0 + 3];
             const F det = fma(u00, u11, -(u01 * u01));
             const bool pd = lq_positive(u00) && lq_positive(det);
             ok = ok && pd;
-            const F id = pd ? -recip(det) : F(0);
+            const F id = pd ? -recip(det) : F(0), i01 = u01 * id;
 #pragma unroll
             for (int r = 0; r < PK; ++r) {
                 const int e = li + L * r;
                 if (e < KE) {
                     const bool x1 = e >= NS + 1;
                     const F own = sm[Mp::H0 + e], other = sm[Mp::H0 + (x1 ? e - (NS + 1) : e + (NS + 1))];
-                    sm[Mp::K0 + e] = fma(x1 ? u00 : u11, own, -(u01 * other)) * id;
+                    sm[Mp::K0 + e] = fma((x1 ? u00 : u11) * id, own, -(i01 * other));
                 }
             }
         }

@@ -10,6 +10,8 @@ import pytest
 
 torch = pytest.importorskip("torch")
 
+from tests.test_gpu_traj import _bicycles
+
 pytestmark = pytest.mark.gpu
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -81,3 +83,20 @@ def test_lq_with_a_huge_control_cost(B, method):
     torch.cuda.synchronize()
     assert int(out["status"][0]) == 0
     assert (out["u"] + 1e308 / 1.5e308).abs().max().item() <= 1e-14
+
+
+def test_trajectory_step_with_a_huge_damping(B, ora):
+    """damp = 0.5e154 at 20 m/s: the 2 x 2 control Hessian is about damp diag(1.01, 5), its
+    determinant 1.26e308 (above 2^1022); 5 damp times the first control's right-hand side,
+    2.2 damp, is beyond the largest number.  One FP64 iteration against the oracle (1e-9,
+    the fixed-iteration parity bound)."""
+    sc = _bicycles([1, 1, 1])
+    sc.u_init[:] = 0.25
+    kw = dict(max_iter=1, eps_pri=0.0, eps_dual=0.0, damp=0.5e154)
+    pb = B.Problem(B.DeviceScene(B.Context(0), sc, torch.float64))
+    rep = pb.solve(**kw)
+    torch.cuda.synchronize()
+    ref = ora.admm_batch(sc, **kw)
+    assert (rep["iters"].cpu().numpy() == ref["iters"]).all() and (rep["status"].cpu().numpy() == ref["status"]).all()
+    for got, want in ((pb.s, ref["s"]), (pb.u, ref["u"])):
+        assert np.abs(got.cpu().numpy() - want).max() <= 1e-9 * (1.0 + np.abs(want).max())
