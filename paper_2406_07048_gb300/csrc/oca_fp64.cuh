@@ -25,4 +25,15 @@ __device__ __forceinline__ double recip(double x) {
 }
 __device__ __forceinline__ float recip(float x) { return 1.0f / x; }
 
+// x > 0 and x finite, and x finite, on the integer pipe (an FP64 compare costs as much as a
+// multiply-add).  A pivot or determinant that overflowed is not taken as positive: the
+// gains would come out 0 or NaN.
+__device__ __forceinline__ bool positive_finite(double x) {
+    const long long b = __double_as_longlong(x);
+    return b > 0 && b < 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool positive_finite(float x) { return x > 0.0f && isfinite(x); }
+__device__ __forceinline__ bool finite(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) != 0x7ff; }
+__device__ __forceinline__ bool finite(float x) { return isfinite(x); }
+
 }  // namespace oca

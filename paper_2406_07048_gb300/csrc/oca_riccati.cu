@@ -186,14 +186,6 @@ __device__ constexpr auto kRicTab = RicBuild<KIND>::template table<PHASE, L>();
 template <int KIND>
 __device__ constexpr auto kRicOut = RicBuild<KIND>::out_map();
 
-// x > 0 and x finite on the integer pipe (an FP64 compare costs as much as a multiply-add)
-__device__ __forceinline__ bool lq_positive(double x) {
-    const long long b = __double_as_longlong(x);
-    return b > 0 && b <= 0x7ff0000000000000ll;
-}
-__device__ __forceinline__ bool lq_positive(float x) { return x > 0.0f; }
-__device__ __forceinline__ bool lq_finite(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) != 0x7ff; }
-__device__ __forceinline__ bool lq_finite(float x) { return isfinite(x); }
 
 // 8- or 4-byte access at a shared-memory byte address
 __device__ __forceinline__ double lds(unsigned at, double) {
@@ -641,7 +633,7 @@ __global__ void __launch_bounds__(32 * kLqWarps) k_traj_lq(LqArgs2<F> a) {
             // pass the largest number where det does not.
             const F u00 = sm[Mp::U0], u01 = sm[Mp::U0 + 1], u11 = sm[Mp::U0 + 3];
             const F det = fma(u00, u11, -(u01 * u01));
-            const bool pd = lq_positive(u00) && lq_positive(det);
+            const bool pd = positive_finite(u00) && positive_finite(det);
             ok = ok && pd;
             const F id = pd ? -recip(det) : F(0), i01 = u01 * id;
 #pragma unroll
@@ -704,7 +696,7 @@ __global__ void __launch_bounds__(32 * kLqWarps) k_traj_lq(LqArgs2<F> a) {
             x = v;
             if (own && t < N) {
                 scr[Mp::sol(N, t) + li] = v;
-                fin = fin && lq_finite(v);
+                fin = fin && finite(v);
             }
             fetch(t + AHEAD, row[d], fv[d]);
         }
@@ -783,7 +775,7 @@ __global__ void __launch_bounds__(128) k_traj_lq4(LqArgs2<F> a) {
                 F col[NU];
 #pragma unroll
                 for (int i = 0; i < NU; ++i) col[i] = __shfl_sync(0xffffffffu, v[i], c);
-                const bool pd = lq_positive(col[c]);
+                const bool pd = positive_finite(col[c]);
                 ok = ok && pd;
                 v[c] *= pd ? recip(col[c]) : F(1);
 #pragma unroll
@@ -835,7 +827,7 @@ __global__ void __launch_bounds__(128) k_traj_lq4(LqArgs2<F> a) {
             x = v;
             if (t < N) {
                 if (!half) scr[Mp::sol(N, t) + i] = v;
-                fin = fin && lq_finite(v);
+                fin = fin && finite(v);
             }
             fetch(t + AHEAD, row[d], fv[d]);
         }

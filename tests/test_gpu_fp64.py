@@ -71,6 +71,19 @@ def test_recip_over_the_range(ops):
     assert got[0] == 0.0 and got[1] == 0.0 and np.isnan(got[2])
 
 
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_classes_over_the_range(ops, dtype):
+    """positive_finite and finite are x > 0 and isfinite, also at both zeros, the smallest
+    and largest numbers, the infinities and NaNs of both signs."""
+    with np.errstate(over="ignore"):
+        x = _operands().astype(dtype)
+    ends = np.array([0.0, np.inf, np.nan, np.finfo(dtype).max, np.finfo(dtype).tiny], dtype=dtype)
+    x = np.concatenate([x, ends, -ends])
+    want = (np.isfinite(x) & (x > 0)) + 2 * np.isfinite(x)
+    got = _apply(ops.run_classes if dtype == np.float64 else ops.run_classes_f32, x, torch.int32)
+    assert (got == want).all()
+
+
 @pytest.mark.parametrize("method", [0, 1])
 def test_lq_with_a_huge_control_cost(B, method):
     """R = 1.5e308, r = 1e308 and controls that reach no state: u = -r / R (the reciprocal of
