@@ -383,7 +383,12 @@ __global__ void __launch_bounds__(kLqGainThreads) k_lq_closed(LqArgs a) {
 }
 
 // ---- closed-loop maps of whole chunks: s_{t0 + L} = G s_{t0} + g over the L steps of
-// chunk blockIdx.x (one product of maps per step)
+// chunk blockIdx.x (one product of maps per step).  Behind G and g a 1 where the rollout may
+// not use the map: a mode that feedback does not reach and that grows by more than
+// kLqMapMax within the chunk.  Its state can be small all the same (0, or held by c), and
+// then G s + g is a difference of large numbers, or inf * 0, where the steps are exact.
+constexpr double kLqMapMax = 65536.0;  // 2^16 of 2^53: at most 1e-11 of the state is lost
+__host__ __device__ inline int lq_map_size(int n) { return n * n + n + 1; }
 template <int CN>
 __global__ void __launch_bounds__(kLqThreads) k_lq_chunk(LqArgs a, double *maps, int L) {
     const int c = blockIdx.x, s = blockIdx.y, tid = threadIdx.x;
@@ -396,7 +401,12 @@ __global__ void __launch_bounds__(kLqThreads) k_lq_chunk(LqArgs a, double *maps,
             cp_async_elem(&Fs[t & 1][e], e < nn ? F0 + (size_t)t * nn + e : f0 + (size_t)t * n + e - nn);
         cp_async_commit();
     };
-    for (int e = tid; e < w; e += kLqThreads) G[0][e] = e < nn ? F0[e] : f0[e - nn];
+    bool far = false;
+    auto put = [&](double *o, int e, double v) {
+        o[e] = v;
+        far = far || !(e < nn ? abs_bits(v) <= abs_bits(kLqMapMax) : finite(v));
+    };
+    for (int e = tid; e < w; e += kLqThreads) put(G[0], e, e < nn ? F0[e] : f0[e - nn]);
     if (L > 1) copy(1);
     for (int t = 1; t < L; ++t) {
         cp_async_wait_all();
@@ -406,16 +416,19 @@ __global__ void __launch_bounds__(kLqThreads) k_lq_chunk(LqArgs a, double *maps,
         double *O = G[t & 1];
         for (int e = tid; e < w; e += kLqThreads) {
             const int i = e < nn ? e / n : e - nn;
-            O[e] = e < nn ? dot_strided<CN>(S + i * n, 1, X + e % n, n, n, 0.0) : dot_strided<CN>(S + i * n, 1, X + nn, 1, n, S[nn + i]);
+            put(O, e, e < nn ? dot_strided<CN>(S + i * n, 1, X + e % n, n, n, 0.0)
+                             : dot_strided<CN>(S + i * n, 1, X + nn, 1, n, S[nn + i]));
         }
     }
-    __syncthreads();
-    double *out = maps + ((size_t)s * gridDim.x + c) * w;
+    far = __syncthreads_or(far);
+    double *out = maps + ((size_t)s * gridDim.x + c) * lq_map_size(n);
     for (int e = tid; e < w; e += kLqThreads) out[e] = G[(L - 1) & 1][e];
+    if (tid == 0) out[w] = far ? 1.0 : 0.0;
 }
 
 // ---- rollout s_{t+1} = F_t s_t + f_t (one warp per chunk and problem): the state at
-// the chunk's start through the maps of the chunks before it, then the chunk's steps.
+// the chunk's start through the maps of the chunks before it (or their steps, where a map
+// may not be used), then the chunk's steps.
 // Lane i and lane 16 + i own s_i and sum one half of its row each; the rows of the next
 // four steps are on their way while a step runs (a step takes about 900 cycles, a load
 // up to 1,500).
@@ -457,12 +470,14 @@ __global__ void __launch_bounds__(32) k_lq_rollout(LqArgs a, const double *maps,
             }
         }
     };
-    const int w = nn + n;
+    const int w = lq_map_size(n), t0 = c * L;
     if (c > 0) {
         const double *m0 = maps + (size_t)s * C * w;
-        roll(m0, w, m0 + nn, w, c, nullptr);
+        bool far = false;  // a map before this chunk that may not be used
+        for (int k2 = lane; k2 < c; k2 += 32) far = far || abs_bits(m0[(size_t)k2 * w + nn + n]) != 0;
+        if (__any_sync(0xffffffffu, far)) roll(a.F + (size_t)s * N * nn, nn, a.f + (size_t)s * N * n, n, t0, nullptr);
+        else roll(m0, w, m0 + nn, w, c, nullptr);
     }
-    const int t0 = c * L;
     const size_t st = (size_t)s * N + t0;
     roll(a.F + st * nn, nn, a.f + st * n, n, min(L, N - t0), a.s + ((size_t)s * (N + 1) + t0 + 1) * n);
 }

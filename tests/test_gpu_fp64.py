@@ -113,3 +113,27 @@ def test_trajectory_step_with_a_huge_damping(B, ora):
     assert (rep["iters"].cpu().numpy() == ref["iters"]).all() and (rep["status"].cpu().numpy() == ref["status"]).all()
     for got, want in ((pb.s, ref["s"]), (pb.u, ref["u"])):
         assert np.abs(got.cpu().numpy() - want).max() <= 1e-9 * (1.0 + np.abs(want).max())
+
+
+@pytest.mark.parametrize("growth,start,N", [(1e20, 0.0, 1024), (3.0, 1.0, 2176)])
+@pytest.mark.parametrize("ns", [2, 12])
+def test_lq_rollout_of_a_mode_that_feedback_does_not_reach(B, growth, start, N, ns):
+    """A mode that grows per step, which no control reaches and no cost sees, at its
+    equilibrium s = growth s + c: step by step it stays there, exactly (small whole numbers).
+    Its map over a chunk of the horizon overflows or passes 2^53."""
+    nu = 4 if ns == 12 else 1
+    f = dict(dtype=torch.float64, device="cuda")
+    A = torch.eye(ns, **f) * 0.5
+    A[0, 0] = growth
+    Bm, c, Q, s0 = torch.zeros(ns, nu, **f), torch.zeros(ns, **f), torch.eye(ns, **f), torch.ones(ns, **f)
+    Bm[1:1 + nu, :] = torch.eye(min(nu, ns - 1), **f)
+    Q[0, 0] = 0.0
+    s0[0], c[0] = start, start * (1.0 - growth)
+    rep = lambda x, k: x.repeat(1, k, *([1] * x.dim()))
+    out = B.lq_solve(B.Context(0), rep(A, N), rep(Bm, N), rep(c, N), rep(Q, N + 1), torch.zeros(1, N + 1, ns, **f),
+                     rep(torch.eye(nu, **f), N), torch.zeros(1, N, nu, **f), s0[None], method=0)
+    torch.cuda.synchronize()
+    assert int(out["status"][0]) == 0
+    assert (out["s"][0, :, 0] == start).all()
+    assert torch.isfinite(out["s"]).all() and torch.isfinite(out["u"]).all()
+    assert out["s"][0, -1, 1:].abs().max().item() < 1e-100
