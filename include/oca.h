@@ -454,6 +454,9 @@ oca_status oca_scale_detect_noalloc(const oca_scene_desc *desc, const oca_model 
  *   (value functions V_t(s) = 0.5 s^T P_t s + p_t^T s + const, each may be NULL),
  *   status [S] int32 (0 solved; 1 a singular R_t, R_t + B^T P B or elimination
  *   pivot, or a non-finite value: that problem's outputs are meaningless).
+ *   R_t (scan) and R_t + B^T P B count as singular when a pivot of the elimination
+ *   (partial pivoting) is not above 1e-300 + 1e-14 of the matrix's own largest entry,
+ *   so that a cost's unit does not matter; the other pivots when not above 1e-300.
  * work: caller-owned device workspace, 256-byte aligned, at least
  * oca_lq_workspace_bytes(...) bytes; nothing is allocated.  ns <= 12, nu <= 4,
  * N <= OCA_MAX_LQ_HORIZON, S <= 65535 (else OCA_ERR_CAPACITY).

@@ -72,7 +72,9 @@ __device__ __forceinline__ unsigned long long abs_bits(double x) {
 // Solve M X = V, M m x m (m <= 4), by Gauss-Jordan elimination with partial pivoting:
 // lane j < m of the warp holds column j of M in v, the lanes from m on the columns of
 // V; on return they hold the columns of X.  False if a pivot is not above 1e-300 +
-// 1e-14 max |M| or M is not finite (1 takes the pivot's place).
+// 1e-14 max |M| or M is not finite (1 takes the pivot's place).  The bound is relative to
+// M alone, for every m: padding M to 4 x 4 with ones, as small systems of 1 to 3 inputs
+// once were, makes 1e-14 the least of it and refuses a control cost of 1e-15.
 __device__ __forceinline__ bool gj_columns(double (&v)[kLqMaxU], int m, int lane) {
     unsigned long long big = 0;
 #pragma unroll

@@ -137,3 +137,20 @@ def test_lq_rollout_of_a_mode_that_feedback_does_not_reach(B, growth, start, N, 
     assert (out["s"][0, :, 0] == start).all()
     assert torch.isfinite(out["s"]).all() and torch.isfinite(out["u"]).all()
     assert out["s"][0, -1, 1:].abs().max().item() < 1e-100
+
+
+@pytest.mark.parametrize("nu", [1, 2, 3, 4])
+@pytest.mark.parametrize("method", [0, 1])
+def test_lq_singular_is_relative_to_the_matrix(B, nu, method):
+    """R = 1e-15 I is solved for every number of inputs (u = -r / R; one division and one
+    product: 1e-15 and the product's rounding), R with equal rows, or 0, is refused."""
+    N, ns = 2, 5
+    z = lambda *shape: torch.zeros(2, *shape, dtype=torch.float64, device="cuda")
+    eye = lambda n, k: torch.eye(n, dtype=torch.float64, device="cuda").repeat(2, k, 1, 1)
+    R = 1e-15 * eye(nu, N)
+    R[1, 1] = 1e-15 if nu > 1 else 0.0
+    out = B.lq_solve(B.Context(0), eye(ns, N), z(N, ns, nu), z(N, ns), eye(ns, N + 1), z(N + 1, ns), R,
+                     z(N, nu) + 3e-15, z(ns) + 1.0, method=method)
+    torch.cuda.synchronize()
+    assert out["status"].cpu().tolist() == [0, 1]
+    assert (out["u"][0] + 3.0).abs().max().item() <= 1e-14
