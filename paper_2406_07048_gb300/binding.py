@@ -347,7 +347,9 @@ class DeviceScene:
         lambda = e_e / b_e with e the part's largest offset (lowest index on
         ties), mu = 0, gamma = 0.  The host only lists the (obstacle, part)
         blocks; filling and transposing the pair array there took most of a
-        closed-loop call (250 of 325 ms for 256 runs of 393,216 pairs)."""
+        closed-loop call (250 of 325 ms for 256 runs of 393,216 pairs).  Like a
+        copy from host arrays it returns when y is there: the call that takes y
+        may run on another stream."""
         sc = self.scene
         y = torch.zeros(sc.ny_max, self.n_pairs, dtype=self.dtype, device=self.device)
         valid = np.arange(sc.fr_max)[None, :] < np.asarray(sc.part_nf)[:, None]
@@ -359,7 +361,9 @@ class DeviceScene:
         part = np.asarray(sc.part_begin)[scen] + k % np.diff(sc.part_begin)[scen]
         n = self.tensor(np.asarray(sc.horizon)[scen], dtype=torch.int64)
         rep = lambda a, dt: torch.repeat_interleave(self.tensor(a[part], dtype=dt), n, output_size=self.n_pairs)
-        return y.scatter_(0, rep(e, torch.int64)[None], rep(val, self.dtype)[None])
+        y.scatter_(0, rep(e, torch.int64)[None], rep(val, self.dtype)[None])
+        torch.cuda.current_stream(self.device).synchronize()
+        return y
 
     @staticmethod
     def to_host_pairs(comp_major: torch.Tensor) -> np.ndarray:

@@ -125,3 +125,14 @@ def test_warps_of_the_pair_and_of_the_lp_kernels(B):
     with pytest.raises(B.OcaError) as e:
         ds.lp_warps = 17
     assert e.value.code == 1
+
+
+def test_cold_start_is_there_when_the_call_returns(B):
+    """The solve that takes the cold start may run on another stream than the one that
+    forms it: nothing of it is pending when cold_y returns."""
+    ds = B.DeviceScene(B.Context(0), synth.config3(n_scen=2048), torch.float32)
+    torch.cuda.synchronize()
+    for stream in (torch.cuda.current_stream(), torch.cuda.Stream()):
+        with torch.cuda.stream(stream):
+            ds.cold_y()
+            assert stream.query()
