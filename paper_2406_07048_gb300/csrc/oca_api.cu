@@ -1085,17 +1085,21 @@ oca_status oca_scene_create(oca_ctx *ctx, const oca_scene_desc *d, oca_scene **o
     std::vector<int> by_horizon(S);
     for (int s = 0; s < S; ++s) by_horizon[s] = s;
     std::stable_sort(by_horizon.begin(), by_horizon.end(), [&](int x, int y) { return sc->meta[x].N > sc->meta[y].N; });
-    // Warps per tile (until oca_scene_set_warps): as many as keep the launch within
-    // `waves` times the warps that an SM holds (16, 12 in FP64 or 3-D, 8 in both, of the
-    // pair kernel; 32 of the LP and margin kernels, by their registers), in counts whose
-    // CTAs fill them, no more than obstacles.  Few tiles then spread their obstacles over
-    // idle SMs, many tiles amortise a warp's set-up over more of them.
+    // Warps per tile (until oca_scene_set_warps, oca_scene_set_lp_warps): as many as keep
+    // the launch within `waves` times the warps that an SM holds (16, 12 in FP64 or 3-D, 8
+    // in both, of the pair kernel; of the LP kernel by its registers and staged columns),
+    // in counts whose CTAs fill them, no more than obstacles.  Few tiles then spread their
+    // obstacles over idle SMs, many tiles amortise a warp's set-up over more of them.
     // Pair kernel, us per launch: 5,660 trailer tiles 706 with 2 (773 with 5), 1,470
     // tiles 208 with 4 (251 with 2, 226 with 8), 345 tiles 74 with 16 (98 with 5), one
     // tile of 4 obstacles in FP64 91 with 4 (264 with 1); in 3-D (equal tiles: one wave)
     // 256 tiles 314 with 6 (389 with 8), 512 tiles 167 with 3 (177 with 8), 16 tiles 195
-    // with 8 (252 with 6).  LP kernel: 2,892 tiles 1,306 with 4 (1,468 with 2), 4 tiles
-    // 100 with 16 (239 with 4); margin kernel: 5,660 tiles 1,107 with 4 (1,134 with 2).
+    // with 8 (252 with 6).  LP kernel (22 warps an SM in FP32 2-D at 20 faces, 11 in FP64,
+    // 16 and 8 in 3-D at 26; L2 flushed): 3 tiles 131 with 16 (264 with 4), 181 tiles 163
+    // with 16 (249 with 8), 1,391 tiles 543 with 4 (656 with 8, 917 with 2), 5,745 tiles
+    // 2,059 with 4 (2,007 with 2, 2,578 with 8); FP64 1,391 tiles 7,699 with 4 (8,020 with
+    // 8, 8,270 with 2); 3-D 256 tiles 1,063 with 16 (1,018 with 8, 1,648 with 4).  The
+    // margin kernel takes the LP's count: 180 to 187 from 4 to 8 at 1,391 tiles.
     auto pick = [&](int per_sm, int most, int least, double waves) {
         const int counts[] = {16, 8, 6, 4, 3, 2, 1};
         for (int w : counts) {
@@ -1108,7 +1112,7 @@ oca_status oca_scene_create(oca_ctx *ctx, const oca_scene_desc *d, oca_scene **o
     const bool one_wave = d->dim == 3 && es == 4;
     sc->W = pick(pair_sm_warps(d->dim, es), pair_max_warps(d->dim, es), one_wave ? 1 : 2, one_wave ? 1.0 : 2.5);
     while (sc->W > 1 && !warps_fit(sc, sc->W)) --sc->W;
-    sc->W_lp = pick(32, 16, 4, 2.5);
+    sc->W_lp = pick(scale_sm_warps(d->dim, es, d->fr_max, d->fo_max), 16, 4, 2.5);
 
     const size_t ts = dsize(d->dtype);
     const int PK = d->dim + d->dim * d->dim;

@@ -18,6 +18,8 @@ int pair_sm_warps(int dim, size_t es);
 // dynamic shared memory of a pair-kernel launch with W warps per tile
 size_t pair_smem_bytes(int dim, size_t es, int W, int mode, int solver, int FR, int FO);
 
+// warps of the scale LP kernel that an SM holds (by its registers and shared memory)
+int scale_sm_warps(int dim, size_t es, int FR, int FO);
 template <typename T>
 cudaError_t launch_scale(const ScaleArgs<T> &a, int dim, int n_tiles, int W, cudaStream_t st);
 

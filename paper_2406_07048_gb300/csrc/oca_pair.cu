@@ -850,6 +850,16 @@ cudaError_t launch_pair(const PairArgs<T> &a, int dim, int mode, int solver, int
     return cudaErrorInvalidValue;
 }
 
+int scale_sm_warps(int dim, size_t es, int FR, int FO) {
+    cudaFuncAttributes at;
+    const void *fn = dim == 2 ? (es == 4 ? (const void *)k_scale<float, 2> : (const void *)k_scale<double, 2>)
+                              : (es == 4 ? (const void *)k_scale<float, 3> : (const void *)k_scale<double, 3>);
+    const size_t smem = es == 4 ? scale_smem_bytes<float>(1, FR, FO) : scale_smem_bytes<double>(1, FR, FO);
+    const int by_smem = (int)(kMaxSmem / smem);
+    if (cudaFuncGetAttributes(&at, fn) != cudaSuccess) return std::max(1, by_smem);
+    return std::max(1, std::min(by_smem, 65536 / (32 * at.numRegs)));
+}
+
 template <typename T>
 cudaError_t launch_scale(const ScaleArgs<T> &a, int dim, int n_tiles, int W, cudaStream_t st) {
     if (n_tiles <= 0) return cudaSuccess;

@@ -136,3 +136,18 @@ def test_cold_start_is_there_when_the_call_returns(B):
         with torch.cuda.stream(stream):
             ds.cold_y()
             assert stream.query()
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+def test_lp_warps_follow_what_an_sm_holds(B, dtype):
+    """More than four warps a tile only while the launch stays within two and a half times
+    the warps whose staged columns (32 lanes x 4 numbers a face) an SM's 227 KB hold."""
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    counts = []
+    for n in (1, 64, 256, 512, 1024):
+        ds = B.DeviceScene(B.Context(0), synth.config3(n_scen=n), dtype)
+        held = 227 * 1024 // (32 * 4 * (ds.scene.fr_max + ds.scene.fo_max) * ds.dtype.itemsize)
+        counts.append(ds.lp_warps)
+        assert ds.lp_warps <= 4 or ds.n_tiles * ds.lp_warps <= 2.5 * n_sm * held
+    # one scene of 12 obstacles, 181 tiles, ..., 2,892 tiles
+    assert counts[:2] == [12, 16] and counts[-1] == 4
