@@ -445,8 +445,9 @@ oca_status oca_scale_detect_noalloc(const oca_scene_desc *desc, const oca_model 
  *                      log2(N) times the recursion's arithmetic for a dependent
  *                      chain of log2(N) rounds instead of N steps (for long
  *                      horizons with few problems).
- * Both then form the gains K_t, k_t of every stage in parallel and roll the
- * closed loop out from s_0 (one warp per problem).
+ * The scan forms the gains K_t, k_t of every stage in parallel, the recursion as
+ * it goes; both then roll the closed loop out from s_0, one warp per problem, or
+ * in chunks of the horizon side by side (few problems of 64 steps and more).
  * Layouts (device, row-major, problem-major):
  *   A [S][N][ns][ns], B [S][N][ns][nu], c [S][N][ns], Q [S][N+1][ns][ns],
  *   q [S][N+1][ns], R [S][N][nu][nu], r [S][N][nu], s0 [S][ns];

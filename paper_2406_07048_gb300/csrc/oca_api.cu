@@ -920,6 +920,8 @@ oca_status dmalloc(P **p, size_t bytes) {
 
 }  // namespace
 
+int oca::ctx_sm_count(const oca_ctx *ctx) { return ctx->n_sm; }
+
 extern "C" {
 
 const char *oca_status_string(oca_status st) {

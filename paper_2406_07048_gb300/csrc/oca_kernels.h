@@ -5,6 +5,9 @@
 
 namespace oca {
 
+// SMs of the context's device
+int ctx_sm_count(const oca_ctx *ctx);
+
 template <typename T>
 cudaError_t launch_pose(const PoseArgs<T> &a, int maxQ, cudaStream_t st);
 

@@ -17,11 +17,15 @@
 //                      (whose A is 0: lam_t = J s_t - eta, the value function
 //                      P_t = J, p_t = -eta) is formed in ceil(log2(N + 1)) rounds
 //                      in which element t takes element t + 2^r, one CTA per
-//                      composition.  The gains K_t, k_t follow per stage in
-//                      parallel, and the rollout s_{t+1} = (A + B K) s + B k + c
-//                      is a dependent chain of matrix-vector products (one warp).
+//                      composition.  The gains K_t, k_t and the closed-loop maps
+//                      A + B K, B k + c follow per stage in parallel.
 //   OCA_LQ_SEQUENTIAL  the backward Riccati recursion over t (one CTA per
-//                      problem), then the same gains and rollout.
+//                      problem), which forms the gains; the closed-loop maps
+//                      follow per stage in parallel.
+//
+// The rollout s_{t+1} = (A + B K) s + B k + c is a dependent chain of matrix-vector
+// products: one warp per problem, or for few problems of 64 steps and more a warp per
+// chunk of steps, started from the products of the maps before its chunk.
 //
 // FP64 throughout.  One CTA per composition: its two elements and the augmented
 // system [I + C1 J2 | A1, b1 + C1 eta2, C1 A2^T] live in shared memory; the system is
@@ -693,7 +697,7 @@ static LqWork lq_work(int n, int m, int N, int S) {
 size_t lq_workspace_bytes(int n, int m, int N, int S) { return lq_work(n, m, N, S).bytes; }
 
 template <int CN, int CM>
-static cudaError_t launch_lq_dims(const LqArgs &a, int method, cudaStream_t st) {
+static cudaError_t launch_lq_dims(const LqArgs &a, int method, int n_sm, cudaStream_t st) {
     const int E = a.N + 1, S = a.S, N = a.N;
     if (method == 0) {
         k_lq_elem<CN, CM><<<dim3(E, S), 32, 0, st>>>(a);
@@ -706,8 +710,9 @@ static cudaError_t launch_lq_dims(const LqArgs &a, int method, cudaStream_t st) 
     } else {
         // a problem's two products have up to 204 and 158 entries: eight warps for the
         // larger dimensions (one entry per thread), two for up to six states
-        if (a.n <= 6) k_lq_seq<CN, CM, 64><<<S, 64, 0, st>>>(a);
-        else k_lq_seq<CN, CM, 256><<<S, 256, 0, st>>>(a);
+        constexpr int NT = CN > 6 ? 256 : 64;
+        if (CN > 0 || a.n <= 6) k_lq_seq<CN, CM, NT><<<S, NT, 0, st>>>(a);
+        else if constexpr (CN == 0) k_lq_seq<0, 0, 256><<<S, 256, 0, st>>>(a);
         if (N > 0) k_lq_closed<CN, CM><<<dim3(N, S), kLqGainThreads, 0, st>>>(a);
     }
     // The rollout's chain: N steps of one warp, or chunks of L steps whose maps are
@@ -715,7 +720,7 @@ static cudaError_t launch_lq_dims(const LqArgs &a, int method, cudaStream_t st) 
     // from about 64 steps on and while their CTAs fit the GPU at once (two per SM): one
     // problem of 256 steps and 12 states 115 -> 41 us.
     const int L = std::max(8, (N + 63) / 64), C = N / L;
-    if (N >= 64 && (long long)S * C <= 2 * 152) {
+    if (N >= 64 && (long long)S * C <= 2 * n_sm) {
         // the last chunk takes the remainder, its map is not needed
         k_lq_chunk<CN><<<dim3(C, S), kLqThreads, 0, st>>>(a, a.buf0, L);
         k_lq_rollout<CN><<<dim3((N + L - 1) / L, S), 32, 0, st>>>(a, a.buf0, C, L);
@@ -728,7 +733,7 @@ static cudaError_t launch_lq_dims(const LqArgs &a, int method, cudaStream_t st) 
 
 cudaError_t launch_lq(int method, int n, int m, int N, int S, const double *A, const double *B, const double *c,
                       const double *Q, const double *q, const double *R, const double *r, const double *s0, double *s,
-                      double *u, double *P, double *p, int *status, void *work, cudaStream_t st) {
+                      double *u, double *P, double *p, int *status, void *work, int n_sm, cudaStream_t st) {
     const LqWork w = lq_work(n, m, N, S);
     unsigned char *wb = static_cast<unsigned char *>(work);
     LqArgs a;
@@ -757,10 +762,10 @@ cudaError_t launch_lq(int method, int n, int m, int N, int S, const double *A, c
     a.f = reinterpret_cast<double *>(wb + w.f);
     k_lq_reset<<<(S + 255) / 256, 256, 0, st>>>(status, S);
     // the dimensions of the three vehicle models have their loops unrolled
-    if (n == 4 && m == 2) return launch_lq_dims<4, 2>(a, method, st);
-    if (n == 5 && m == 2) return launch_lq_dims<5, 2>(a, method, st);
-    if (n == 12 && m == 4) return launch_lq_dims<12, 4>(a, method, st);
-    return launch_lq_dims<0, 0>(a, method, st);
+    if (n == 4 && m == 2) return launch_lq_dims<4, 2>(a, method, n_sm, st);
+    if (n == 5 && m == 2) return launch_lq_dims<5, 2>(a, method, n_sm, st);
+    if (n == 12 && m == 4) return launch_lq_dims<12, 4>(a, method, n_sm, st);
+    return launch_lq_dims<0, 0>(a, method, n_sm, st);
 }
 
 }  // namespace oca
@@ -787,6 +792,6 @@ extern "C" oca_status oca_lq_solve(oca_ctx *ctx, int32_t method, int32_t ns, int
     if (work_bytes < (int64_t)lq_workspace_bytes(ns, nu, N, n_problems)) return OCA_ERR_CAPACITY;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const cudaError_t e = launch_lq(method == OCA_LQ_SCAN ? 0 : 1, ns, nu, N, n_problems, A, B, c, Q, q, R, r, s0, s,
-                                    u, P, p, status, work, st);
+                                    u, P, p, status, work, ctx_sm_count(ctx), st);
     return e == cudaSuccess ? OCA_OK : OCA_ERR_CUDA;
 }
