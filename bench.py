@@ -441,7 +441,8 @@ def traj_roofline(scene, stages, traj_ms, fp64):
     f_stage = ric_flops_per_stage(scene.model.ns, scene.model.nu)
     ach = f_stage * stages / (traj_ms / 1e3) / 1e9
     return {"bound": "fp64", "achieved": ach, "peak": fp64, "unit": "GFLOP/s", "frac": ach / fp64 if fp64 > 0 else None,
-            "kernel": "k_traj_lq (FP64 backward Riccati recursion + forward sweep; launch time includes the stage assembly and update)",
+            "kernel": ("k_traj_lq4" if scene.dim == 3 else "k_traj_lq") +
+                      " (FP64 backward Riccati recursion + forward sweep; launch time includes the stage assembly and update)",
             "flops_per_stage": f_stage, "stages": stages,
             "peak_source": "measured on this GPU (oca_fp64_peak: FP64 FMA microbenchmark)"}
 

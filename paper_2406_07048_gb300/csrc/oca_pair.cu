@@ -63,10 +63,10 @@ __global__ void k_pose(PoseArgs<T> a) {
 // Launch bound of the pair kernel, which sets its registers and with them the resident
 // warps per SM: 512 threads for the FP32 2-D kernel, whose state fits 128 registers
 // without spilling (16 warps); 384 for the FP64 2-D kernel (about 165 registers, 12
-// warps) and for the FP32 3-D kernel (4 x 4 Newton systems, up to 8 robot faces: 168
-// registers with a few spilled, 12 warps -- 64 quadrotor scenes 376 -> 314 us per launch
-// against 245 registers and 8 warps; 128 registers spill too much: 374 us); 256 for the
-// FP64 3-D kernel.
+// warps) and for the FP32 3-D kernel (4 x 4 Newton systems, up to 8 robot faces: 165 to 168
+// registers, none spilled with prox > 0, 12 warps -- 64 quadrotor scenes 376 -> 314 us per
+// launch against 245 registers and 8 warps; 128 registers spill: 374 us); 256 for the FP64
+// 3-D kernel.
 #ifndef OCA_PAIR_MAX_THREADS_2D
 #define OCA_PAIR_MAX_THREADS_2D 512
 #endif

@@ -1,6 +1,7 @@
 // Trajectory step of the ADMM (Sec. IV-B eqn:ADMM_state_updates): the LQ
-// stage terms and the Riccati factorisation and sweep, shared by the
-// forward kernel (oca_riccati.cu) and the adjoint kernel (oca_adjoint.cu).
+// stage terms, shared by the forward and the reverse step (oca_riccati.cu,
+// oca_adjoint.cu), and the dense Riccati factorisation and sweep of the
+// 12-state model's reverse step (the others run slot lists: oca_ricprog.cuh).
 //
 // The LQ problem of one scenario (one SQP step at the linearisation point
 // (s^j, u^j)):
@@ -296,70 +297,55 @@ __device__ __forceinline__ F ric_stage_elem(const F *scr, int N, int t, int e) {
 // inverse of a symmetric positive-definite n x n matrix (n <= 4), in registers
 template <typename F, int NU>
 __device__ __forceinline__ bool spd_inverse(const F (&U)[NU][NU], F (&X)[NU][NU]) {
-    if constexpr (NU == 2) {
-        const F det = U[0][0] * U[1][1] - U[0][1] * U[0][1];
-        if (!(U[0][0] > F(0)) || !(det > F(0))) {
-            // not positive definite: X = 0 (the gains of this stage vanish; the
-            // caller reports the failure), never values left from before
-            X[0][0] = X[0][1] = X[1][0] = X[1][1] = F(0);
-            return false;
+    // U = L D L^T (L unit lower triangular: no square roots on the
+    // dependent chain), then X = L^-T D^-1 L^-1; U is positive definite
+    // iff every pivot d_c is positive
+    F L[NU][NU], dg[NU], idg[NU];
+    bool ok = true;
+#pragma unroll
+    for (int c = 0; c < NU; ++c) {
+        F dc = U[c][c];
+#pragma unroll
+        for (int k = 0; k < c; ++k) dc -= L[c][k] * L[c][k] * dg[k];
+        ok &= dc > F(0);
+        dc = dc > F(0) ? dc : F(1);
+        dg[c] = dc;
+        idg[c] = F(1) / dc;
+#pragma unroll
+        for (int r = c + 1; r < NU; ++r) {
+            F acc = U[r][c];
+#pragma unroll
+            for (int k = 0; k < c; ++k) acc -= L[r][k] * L[c][k] * dg[k];
+            L[r][c] = acc * idg[c];
         }
-        const F id = F(1) / det;
-        X[0][0] = U[1][1] * id;
-        X[1][1] = U[0][0] * id;
-        X[0][1] = X[1][0] = -U[0][1] * id;
-        return true;
-    } else {
-        // U = L D L^T (L unit lower triangular: no square roots on the
-        // dependent chain), then X = L^-T D^-1 L^-1; U is positive definite
-        // iff every pivot d_c is positive
-        F L[NU][NU], dg[NU], idg[NU];
-        bool ok = true;
+    }
+    // Z = L^-1 (unit lower triangular)
+    F Z[NU][NU];
 #pragma unroll
-        for (int c = 0; c < NU; ++c) {
-            F dc = U[c][c];
+    for (int c = 0; c < NU; ++c)
 #pragma unroll
-            for (int k = 0; k < c; ++k) dc -= L[c][k] * L[c][k] * dg[k];
-            ok &= dc > F(0);
-            dc = dc > F(0) ? dc : F(1);
-            dg[c] = dc;
-            idg[c] = F(1) / dc;
-#pragma unroll
-            for (int r = c + 1; r < NU; ++r) {
-                F acc = U[r][c];
-#pragma unroll
-                for (int k = 0; k < c; ++k) acc -= L[r][k] * L[c][k] * dg[k];
-                L[r][c] = acc * idg[c];
-            }
-        }
-        // Z = L^-1 (unit lower triangular)
-        F Z[NU][NU];
-#pragma unroll
-        for (int c = 0; c < NU; ++c)
-#pragma unroll
-            for (int r = 0; r < NU; ++r) {
-                if (r < c) {
-                    Z[r][c] = F(0);
-                } else if (r == c) {
-                    Z[r][c] = F(1);
-                } else {
-                    F acc = F(0);
-#pragma unroll
-                    for (int k = c; k < r; ++k) acc -= L[r][k] * Z[k][c];
-                    Z[r][c] = acc;
-                }
-            }
-#pragma unroll
-        for (int i = 0; i < NU; ++i)
-#pragma unroll
-            for (int j = 0; j <= i; ++j) {
+        for (int r = 0; r < NU; ++r) {
+            if (r < c) {
+                Z[r][c] = F(0);
+            } else if (r == c) {
+                Z[r][c] = F(1);
+            } else {
                 F acc = F(0);
 #pragma unroll
-                for (int k = 0; k < NU; ++k) acc += Z[k][i] * idg[k] * Z[k][j];
-                X[i][j] = X[j][i] = acc;
+                for (int k = c; k < r; ++k) acc -= L[r][k] * Z[k][c];
+                Z[r][c] = acc;
             }
-        return ok;
-    }
+        }
+#pragma unroll
+    for (int i = 0; i < NU; ++i)
+#pragma unroll
+        for (int j = 0; j <= i; ++j) {
+            F acc = F(0);
+#pragma unroll
+            for (int k = 0; k < NU; ++k) acc += Z[k][i] * idg[k] * Z[k][j];
+            X[i][j] = X[j][i] = acc;
+        }
+    return ok;
 }
 
 // one warp runs the recursion
