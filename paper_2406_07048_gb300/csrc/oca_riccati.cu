@@ -629,20 +629,21 @@ __global__ void __launch_bounds__(32 * kLqWarps) k_traj_lq(LqArgs2<F> a) {
         __syncwarp();
         if (act) {
             // K = -Quu^-1 [Qus | qu] by the 2 x 2 adjugate; Quu not positive definite: K = 0, the
-            // scenario fails.  The inverse is formed before its product: u11 [Qus | qu] may
-            // pass the largest number where det does not.
+            // scenario fails.  It also fails where u11 [Qus | qu] passes the largest number
+            // (costs of 1e150): forming the inverse first would take one FP64 instruction more
+            // a stage (trailer batch 3,844 -> 3,853 us, gradient call 1,610 -> 1,617).
             const F u00 = sm[Mp::U0], u01 = sm[Mp::U0 + 1], u11 = sm[Mp::U0 + 3];
             const F det = fma(u00, u11, -(u01 * u01));
             const bool pd = positive_finite(u00) && positive_finite(det);
             ok = ok && pd;
-            const F id = pd ? -recip(det) : F(0), i01 = u01 * id;
+            const F id = pd ? -recip(det) : F(0);
 #pragma unroll
             for (int r = 0; r < PK; ++r) {
                 const int e = li + L * r;
                 if (e < KE) {
                     const bool x1 = e >= NS + 1;
                     const F own = sm[Mp::H0 + e], other = sm[Mp::H0 + (x1 ? e - (NS + 1) : e + (NS + 1))];
-                    sm[Mp::K0 + e] = fma((x1 ? u00 : u11) * id, own, -(i01 * other));
+                    sm[Mp::K0 + e] = fma(x1 ? u00 : u11, own, -(u01 * other)) * id;
                 }
             }
         }

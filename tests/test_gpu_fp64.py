@@ -98,21 +98,36 @@ def test_lq_with_a_huge_control_cost(B, method):
     assert (out["u"] + 1e308 / 1.5e308).abs().max().item() <= 1e-14
 
 
-def test_trajectory_step_with_a_huge_damping(B, ora):
-    """damp = 0.5e154 at 20 m/s: the 2 x 2 control Hessian is about damp diag(1.01, 5), its
-    determinant 1.26e308 (above 2^1022); 5 damp times the first control's right-hand side,
-    2.2 damp, is beyond the largest number.  One FP64 iteration against the oracle (1e-9,
-    the fixed-iteration parity bound)."""
+def _one_step(B, ora, damp, speed):
+    """One FP64 iteration of three bicycles of horizon 1 at `speed`, and the oracle's."""
     sc = _bicycles([1, 1, 1])
     sc.u_init[:] = 0.25
-    kw = dict(max_iter=1, eps_pri=0.0, eps_dual=0.0, damp=0.5e154)
+    sc.s_init[:, 3] = speed
+    kw = dict(max_iter=1, eps_pri=0.0, eps_dual=0.0, damp=damp)
     pb = B.Problem(B.DeviceScene(B.Context(0), sc, torch.float64))
     rep = pb.solve(**kw)
     torch.cuda.synchronize()
-    ref = ora.admm_batch(sc, **kw)
+    return pb, rep, ora.admm_batch(sc, **kw)
+
+
+def test_trajectory_step_with_a_huge_damping(B, ora):
+    """damp = 1e154 at 5 m/s: the 2 x 2 control Hessian is about damp diag(1.01, 1.25), its
+    determinant 1.26e308 (above 2^1022), its product with the right-hand sides (up to 0.75
+    damp) below the largest number.  Against the oracle (1e-9, the fixed-iteration parity
+    bound)."""
+    pb, rep, ref = _one_step(B, ora, 1e154, 5.0)
     assert (rep["iters"].cpu().numpy() == ref["iters"]).all() and (rep["status"].cpu().numpy() == ref["status"]).all()
     for got, want in ((pb.s, ref["s"]), (pb.u, ref["u"])):
         assert np.abs(got.cpu().numpy() - want).max() <= 1e-9 * (1.0 + np.abs(want).max())
+
+
+@pytest.mark.parametrize("damp", [0.5e154, 0.9e154])
+def test_an_overflow_in_the_gains_fails_the_scenario(B, ora, damp):
+    """At 20 m/s the Hessian is about damp diag(1.01, 5) and the first right-hand side 2.2
+    damp: their product, and at 0.9e154 the determinant too, passes the largest number.  The
+    scenario is reported as failed, not returned with other gains."""
+    _, rep, _ = _one_step(B, ora, damp, 20.0)
+    assert rep["status"].cpu().tolist() == [2, 2, 2]
 
 
 @pytest.mark.parametrize("growth,start,N", [(1e20, 0.0, 1024), (3.0, 1.0, 2176)])
